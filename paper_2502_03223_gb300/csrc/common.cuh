@@ -9,6 +9,7 @@
 #include <string.h>
 
 #include "sacra2d.h"
+#include "softfp.cuh"
 
 namespace sacra {
 
@@ -216,6 +217,19 @@ __device__ __forceinline__ double to_f64(T v) {
   else return v;
 }
 
+// ------------------------------------------------------------------ quotients and roots in arithmetic T
+//
+// FP64: on the integer units (softfp.cuh), 15 to 20 SM cycles per warp instead
+// of 90 to 146 on the FP64 pipe; FP32: the hardware forms.
+__device__ __forceinline__ double t_div(double a, double b) { return sf::sdiv(a, b); }
+__device__ __forceinline__ double t_rcp(double a) { return sf::srcp(a); }
+__device__ __forceinline__ double t_sqrt(double a) { return sf::ssqrt(a); }
+__device__ __forceinline__ double t_rsqrt(double a) { return sf::srsqrt(a); }
+__device__ __forceinline__ float t_div(float a, float b) { return a / b; }
+__device__ __forceinline__ float t_rcp(float a) { return 1.0f / a; }
+__device__ __forceinline__ float t_sqrt(float a) { return sqrtf(a); }
+__device__ __forceinline__ float t_rsqrt(float a) { return rsqrtf(a); }
+
 // ------------------------------------------------------------------ small tensor helpers
 
 template <typename T>
@@ -230,7 +244,7 @@ __device__ inline Sym3T<T> s3inv(const Sym3T<T> &g, T *detp) {
   const T cxy = g.xz * g.yz - g.xy * g.zz;
   const T cxz = g.xy * g.yz - g.xz * g.yy;
   const T det = g.xx * cxx + g.xy * cxy + g.xz * cxz;
-  const T id = T(1) / det;
+  const T id = t_rcp(det);
   Sym3T<T> r;
   r.xx = cxx * id; r.xy = cxy * id; r.xz = cxz * id;
   r.yy = (g.xx * g.zz - g.xz * g.xz) * id;
@@ -315,7 +329,7 @@ __device__ inline T eos_p(const DevParams &p, T rho, T eps) {
 }
 template <typename T>
 __device__ inline T eos_eps(const DevParams &p, T rho, T P) {
-  return eos_ec(p, rho) + (P - eos_pc(p, rho)) / (pv<T>(p.Gamma_th - 1.0, p.fGth1) * rho);
+  return eos_ec(p, rho) + t_div(P - eos_pc(p, rho), pv<T>(p.Gamma_th - 1.0, p.fGth1) * rho);
 }
 // c_s^2 rho h = Gamma P_cold + Gamma_th P_th, clamped to [0, 1)
 template <typename T>
@@ -343,11 +357,11 @@ __device__ inline void prim_to_cons(const DevParams &p, const double pr[NPRIM], 
   double w = 1.0;
   if (u[0] != 0.0 || u[1] != 0.0 || u[2] != 0.0) {
     const Sym3 gi = s3inv(gt, (double *)nullptr);
-    w = sqrt(1.0 + W * W * s3quad(gi, u, u));
+    w = t_sqrt(1.0 + W * W * s3quad(gi, u, u));
   }
   const double rho = pr[pRHO], P = pr[pP];
-  const double rhw = rho * (1.0 + pr[pEPS] + P / rho) * w;
-  const double psi6 = 1.0 / (W * W * W);
+  const double rhw = rho * (1.0 + pr[pEPS] + t_div(P, rho)) * w;
+  const double psi6 = sf::sdiv_rn(1.0, W * W * W);   // rounded as the division: D = q W^3 meets rho_atm here
   q[0] = psi6 * rho * w;
   q[1] = psi6 * rhw * u[0];
   q[2] = psi6 * rhw * u[1] * (p.geometry == SACRA_CYLINDRICAL ? x : 1.0);
@@ -365,18 +379,18 @@ struct C2pD {
 // h = (1 + eps)(1 + a), a = P / (rho (1 + eps)), is formed as 1 + eps + P / rho.
 template <bool COLD>
 __device__ inline double c2p_fun(const DevParams &p, double z, C2pD D, double qq, double r) {
-  const double w2 = 1.0 + z * z, iw = rsqrt(w2);   // 1 / w: rho = D / w without a division
+  const double w2 = 1.0 + z * z, iw = t_rsqrt(w2);   // 1 / w: rho = D / w without a division
   const double w = w2 * iw;
   const double rho = D.v * iw, irho = w * D.inv;
   if (COLD) {
     const double hc = 1.0 + eos_ec(p, rho) + eos_pc(p, rho) * irho;
-    return z - r / hc;
+    return z - t_div(r, hc);
   }
-  double eps = w * qq - z * r + z * z / (1.0 + w);
+  double eps = w * qq - z * r + t_div(z * z, 1.0 + w);
   const double emin = eos_ec(p, rho);
   if (eps < emin) eps = emin;
   const double P = eos_p(p, rho, eps);
-  return z - r / (1.0 + eps + P * irho);
+  return z - t_div(r, 1.0 + eps + P * irho);
 }
 
 // Illinois bracketing iteration from the bracket [a, b] with the master
@@ -396,7 +410,7 @@ __device__ double illinois_from(const DevParams &p, double a, double fa, double 
   double c = a;
   for (int it = 1; it <= p.c2p_maxit; ++it) {
     *its = it;
-    c = (a * fb - b * fa) / (fb - fa);
+    c = t_div(a * fb - b * fa, fb - fa);
     const double fc = c2p_fun<COLD>(p, c, D, qq, r);
     if (fc == 0.0) return c;
     if (fc * fb > 0.0) {
@@ -439,7 +453,7 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
   const double W3 = W * W * W;
   const double D = q[0] * W3;
   double S[3] = {q[1] * W3, q[2] * W3, q[3] * W3};
-  if (p.geometry == SACRA_CYLINDRICAL) S[1] /= x;
+  if (p.geometry == SACRA_CYLINDRICAL) S[1] = t_div(S[1], x);
   const double E = q[4] * W3;
   if (!(D > 0.0) || !(E > 0.0) || !isfinite(D) || !isfinite(E) || !isfinite(S[0]) || !isfinite(S[1]) ||
       !isfinite(S[2])) {
@@ -455,7 +469,8 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
     return ST_ATM;
   }
   int st = 0;
-  double r = sqrt(W * W * s3quad(gi, S, S)) / D;
+  const double iD = t_rcp(D);
+  double r = t_div(t_sqrt(W * W * s3quad(gi, S, S)), D);
   if (p.adiabatic) {
     // "adiabatic" EOS (Sec. III): zero temperature, the energy equation is
     // discarded: the cold recovery from D and S_i alone, the Lorentz factor
@@ -467,12 +482,12 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
       st |= ST_KRESCALE;
     }
     int its, ok;
-    const double z = illinois<true>(p, 0.0, r, C2pD{D, 1.0 / D}, 0.0, r, &its, &ok);
+    const double z = illinois<true>(p, 0.0, r, C2pD{D, iD}, 0.0, r, &its, &ok);
     if (!ok) st |= ST_NOCONV;
-    const double w = sqrt(1.0 + z * z);
-    const double rho = D / w;
+    const double iw = t_rsqrt(1.0 + z * z);
+    const double rho = D * iw;
     const double eps = eos_ec(p, rho), P = eos_pc(p, rho);
-    const double iDh = 1.0 / (D * (1.0 + eps + P / rho));
+    const double iDh = t_rcp(D * (1.0 + eps + t_div(P, rho)));
     pr[pRHO] = rho;
     pr[pEPS] = eps;
     pr[pP] = P;
@@ -486,9 +501,9 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
     prim_to_cons(p, pr, W, gt, x, q);
     return st;
   }
-  const C2pD Dd{D, 1.0 / D};
-  const double qq = E / D - 1.0;
-  double k = r / (1.0 + qq);
+  const C2pD Dd{D, iD};
+  const double qq = sf::sdiv_rn(E, D) - 1.0;   // E / D - 1 is near the cold curve's eps: rounded as the division
+  double k = t_div(r, 1.0 + qq);
   const double kmax = p.c2p_kmax;
   if (k > kmax) {
     const double s = kmax / k;
@@ -497,8 +512,8 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
     k = kmax;
     st |= ST_KRESCALE;
   }
-  const double zlo = 0.5 * k * rsqrt(1.0 - 0.25 * k * k);
-  const double zhi = k * rsqrt(1.0 - k * k);
+  const double zlo = 0.5 * k * t_rsqrt(1.0 - 0.25 * k * k);
+  const double zhi = k * t_rsqrt(1.0 - k * k);
   int its, ok;
   double z = 0.0;
   bool solved = false;
@@ -546,22 +561,22 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
     atomicAdd(p.c2p_stats + 3, 1ull);
   }
   if (!ok) st |= ST_NOCONV;
-  double w = sqrt(1.0 + z * z);
-  double rho = D / w;
-  double eps = w * qq - z * r + z * z / (1.0 + w);
+  double w = t_sqrt(1.0 + z * z);
+  double rho = t_div(D, w);
+  double eps = w * qq - z * r + t_div(z * z, 1.0 + w);
   double P;
   if (eps < eos_ec(p, rho)) {
     z = illinois<true>(p, 0.0, r, Dd, qq, r, &its, &ok);
     if (!ok) st |= ST_NOCONV;
-    w = sqrt(1.0 + z * z);
-    rho = D / w;
+    w = t_sqrt(1.0 + z * z);
+    rho = t_div(D, w);
     eps = eos_ec(p, rho);
     P = eos_pc(p, rho);
     st |= ST_COLD;
   } else {
     P = eos_p(p, rho, eps);
   }
-  const double iDh = 1.0 / (D * (1.0 + eps + P / rho));
+  const double iDh = t_rcp(D * (1.0 + eps + t_div(P, rho)));
   pr[pRHO] = rho;
   pr[pEPS] = eps;
   pr[pP] = P;
@@ -653,12 +668,12 @@ __device__ inline void sr_state(const DevParams &p, T rho, T P, T Poff, T u0, T 
     P = Pc;
   }
   // the EOS quantities of eos_eps and eos_cs2 with one reciprocal of rho and of w
-  const T w = sqrt(T(1) + u0 * u0 + u1 * u1 + u2 * u2);
-  const T iw = T(1) / w, irho = T(1) / rho;
+  const T w = t_sqrt(T(1) + u0 * u0 + u1 * u1 + u2 * u2);
+  const T iw = t_rcp(w), irho = t_rcp(rho);
   const T pc = eos_pc(p, rho);
   const T eps = eos_ec(p, rho) + (P - pc) * irho * pv<T>(p.ith1, p.fith1);
   const T h = T(1) + eps + P * irho;
-  T c2 = (eos_gc(p, rho) * pc + pv<T>(p.Gamma_th, p.fGamma_th) * (P - pc)) * irho / h;
+  T c2 = t_div((eos_gc(p, rho) * pc + pv<T>(p.Gamma_th, p.fGamma_th) * (P - pc)) * irho, h);
   if (!(c2 > T(0))) c2 = T(0);
   if (c2 >= T(1)) c2 = sizeof(T) == 8 ? T(1.0 - 1e-15) : T(1.0f - 1e-6f);
   const T rhw = rho * h * w;          // rho h w^2 v = rho h w u
@@ -670,8 +685,8 @@ __device__ inline void sr_state(const DevParams &p, T rho, T P, T Poff, T u0, T 
   s.vx = v0;
   const T vv = v0 * v0 + v1 * v1 + v2 * v2;
   T disc = c2 * (T(1) - vv) * (T(1) - vv * c2 - v0 * v0 * (T(1) - c2));
-  disc = disc < T(0) ? T(0) : sqrt(disc);
-  const T den = T(1) / (T(1) - vv * c2);
+  disc = disc < T(0) ? T(0) : t_sqrt(disc);
+  const T den = t_rcp(T(1) - vv * c2);
   s.lm = (v0 * (T(1) - c2) - disc) * den;
   s.lp = (v0 * (T(1) - c2) + disc) * den;
 }
@@ -718,8 +733,8 @@ __device__ inline int face_flux(const DevParams &p, int dir, const T pl[5], cons
     uR[0] = pr[3]; uR[1] = pr[1]; uR[2] = pr[2];
   }
   const Sym3T<T> mi = s3inv(m, (T *)nullptr);
-  const T Bh = rsqrt(mi.xx);                 // 1/sqrt(gt^xx)
-  const T Ch = rsqrt(m.zz);                  // 1/sqrt(gt_zz)
+  const T Bh = t_rsqrt(mi.xx);                 // 1/sqrt(gt^xx)
+  const T Ch = t_rsqrt(m.zz);                  // 1/sqrt(gt_zz)
   const T Dh = Bh * Ch;
   // tetrad components of u: e_(a)^i u_i with the contravariant legs
   //   e_x = W B (gt^xx, gt^xy, gt^xz), e_y = W D (0, gt_zz, -gt_yz), e_z = W C (0, 0, 1)
@@ -746,7 +761,7 @@ __device__ inline int face_flux(const DevParams &p, int dir, const T pl[5], cons
   const T lamL = fmin(L.lm, R.lm);
   const T lamR = fmax(L.lp, R.lp);
   const T sgxx = W * (mi.xx * Bh);           // W sqrt(gt^xx)
-  const T vint = bn / (alpha * sgxx);
+  const T vint = t_div(bn, alpha * sgxx);
 
   T F[5];
   int fb = 0;
@@ -758,7 +773,7 @@ __device__ inline int face_flux(const DevParams &p, int dir, const T pl[5], cons
     } else if (lamR <= vint) {
       for (int n = 0; n < 5; ++n) F[n] = fR[n] - vint * qR[n];
     } else {
-      const T idl = T(1) / (lamR - lamL);
+      const T idl = t_rcp(lamR - lamL);
       // HLL state and flux, only the components the contact speed needs
       const T Eh = (lamR * qR[4] - lamL * qL[4] + fL[4] - fR[4]) * idl;
       const T Sh = (lamR * qR[1] - lamL * qL[1] + fL[1] - fR[1]) * idl;
@@ -769,7 +784,7 @@ __device__ inline int face_flux(const DevParams &p, int dir, const T pl[5], cons
       bool bad = !(disc >= T(0));
       T lamc = T(0), Pc = T(0);
       if (!bad) {
-        lamc = T(2) * Sh / (bb + sqrt(disc));     // minus root, cancellation free
+        lamc = t_div(T(2) * Sh, bb + t_sqrt(disc));     // minus root, cancellation free
         Pc = FSh - lamc * FEh;
         bad = !(lamc >= lamL && lamc <= lamR) || !((kDelta ? Pc + pref : Pc) > T(0));
       }
@@ -779,7 +794,7 @@ __device__ inline int face_flux(const DevParams &p, int dir, const T pl[5], cons
         const T *qK = left ? qL : qR;
         const T *fK = left ? fL : fR;
         const T lamK = left ? lamL : lamR;
-        const T iden = T(1) / (lamK - lamc);
+        const T iden = t_rcp(lamK - lamc);
         if constexpr (kDelta) {
           // q* - q_K = [(lambda_c - v_K) q_K + (P_c - P_K) (0, 1, 0, 0, lambda_c)
           //             + P_K (lambda_c - v_K) (0, 0, 0, 0, 1)] / (lambda_K - lambda_c)
@@ -820,7 +835,7 @@ __device__ inline int face_flux(const DevParams &p, int dir, const T pl[5], cons
   }
   // back to the Eulerian frame with the covariant legs e_(a)_i:
   //   e_x = (B/W)(1,0,0), e_y = (D/W)(-gt^xy, gt^xx, 0), e_z = (C/W)(gt_xz, gt_yz, gt_zz)
-  const T iW = T(1) / W;
+  const T iW = t_rcp(W);
   const T pre = alpha * (iW * iW * iW) * sgxx;
   const T S0 = iW * (Bh * F[1] - Dh * mi.xy * F[2] + Ch * m.xz * F[3]);
   const T S1 = iW * (Dh * mi.xx * F[2] + Ch * m.yz * F[3]);

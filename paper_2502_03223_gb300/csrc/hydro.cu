@@ -305,7 +305,7 @@ __device__ inline bool flux_f32(const Lev &L, const DevParams &p, const double *
   const size_t P = L.P;
   const int id = cid(L, j, k);
   const double aj64 = U[(size_t)fAL * P + id], Wj64 = U[(size_t)fW * P + id], Pj = L.prim[(size_t)pP * P + id];
-  out[n] += aj64 * Pj / (Wj64 * Wj64 * Wj64);
+  out[n] += t_div(aj64 * Pj, Wj64 * Wj64 * Wj64);
   return true;
 }
 
@@ -496,7 +496,7 @@ __device__ __forceinline__ void hydro_rhs_cell(const Lev &L, const DevParams &p,
   const int sz = L.px;
   const bool cyl = p.geometry == SACRA_CYLINDRICAL;
   const double xd = (j - 0.5) * L.dx;
-  const double ivol = 1.0 / (cyl ? xd * L.dx * L.dz : L.dx * L.dz);
+  const double ivol = t_rcp(cyl ? xd * L.dx * L.dz : L.dx * L.dz);
   double div[NCONS];
 #pragma unroll
   for (int v = 0; v < NCONS; ++v) {
@@ -522,15 +522,15 @@ __device__ __forceinline__ void hydro_rhs_cell(const Lev &L, const DevParams &p,
   for (int f = 0; f < NPRIM; ++f) pr[f] = ld_as<T>(L.prim[(size_t)f * P + id]);
   const T rho = pr[pRHO], Pp = pr[pP];
   const T u[3] = {pr[pUX], pr[pUY], pr[pUZ]};
-  const T w = sqrt(T(1) + W * W * s3quad(gi, u, u));
-  const T iw = T(1) / w;
-  const T rhw2 = rho * (T(1) + pr[pEPS] + Pp / rho) * w * w;
+  const T w = t_sqrt(T(1) + W * W * s3quad(gi, u, u));
+  const T iw = t_rcp(w);
+  const T rhw2 = rho * (T(1) + pr[pEPS] + t_div(Pp, rho)) * w * w;
   const T vd[3] = {u[0] * iw, u[1] * iw, u[2] * iw};
   T vu[3];
   s3vec(gi, vd, vu);
   vu[0] *= W * W; vu[1] *= W * W; vu[2] *= W * W;
   const T vv = vd[0] * vu[0] + vd[1] * vu[1] + vd[2] * vu[2];
-  const T iW = T(1) / W, iW3 = iW * iW * iW;
+  const T iW = t_rcp(W), iW3 = iW * iW * iW;
   // gt^ac v_c, used in v_a v_b d gt^ab = -(gt^ac v_c)(gt^bd v_d) d gt_cd
   T gv[3];
   s3vec(gi, vd, gv);
@@ -565,8 +565,8 @@ __device__ __forceinline__ void hydro_rhs_cell(const Lev &L, const DevParams &p,
   }
   T geo = T(0);
   if (cyl) {
-    const T vbary = vu[1] - ld(fBY) / al;
-    geo = al * iW3 * (rhw2 * vd[1] * vbary + Pp) / x;
+    const T vbary = vu[1] - t_div(ld(fBY), al);
+    geo = t_div(al * iW3 * (rhw2 * vd[1] * vbary + Pp), x);
   }
   // K^ij S_ij = rho h w^2 K_ij v^i v^j + P gamma^ij K_ij, K_ij = (At_ij + gt_ij K/3) / W^2
   T K;

@@ -94,7 +94,7 @@ __device__ inline void geo_ricci(const Z4cIn<T> &z, Geo<T> &G) {
   for (int a = 0; a < 6; ++a) DDW[a] = z.ddW[a] - (G.G2[0][a] * z.dW[0] + G.G2[1][a] * z.dW[1] + G.G2[2][a] * z.dW[2]);
   const T trDDW = gi.xx * DDW[0] + gi.yy * DDW[3] + gi.zz * DDW[5] + T(2.0) * (gi.xy * DDW[1] + gi.xz * DDW[2] + gi.yz * DDW[4]);
   const T dW2 = s3quad(gi, z.dW, z.dW);
-  const T iW = T(1.0) / z.W;
+  const T iW = t_rcp(z.W);
   // gt^lm (Gt^k_li Gt_{j,km} + Gt^k_lj Gt_{i,km} + Gt^k_im Gt_{k,lj}) with the last
   // index of Gt_{j,km} raised once, M[j][k][l] = gt^lm Gt_{j,km}: the first two
   // terms are Q_ij + Q_ji with Q_ij = Gt^k_li M[j][k][l], the third Gt^k_im M[k][j][m]
@@ -152,12 +152,12 @@ __device__ inline void geo_ricci(const Z4cIn<T> &z, Geo<T> &G) {
 template <typename T>
 __device__ inline void matter(const T pr[NPRIM], T W, const Sym3T<T> &g, const Sym3T<T> &gi, T &E, T S[3], T Sij[6]) {
   const T u[3] = {pr[pUX], pr[pUY], pr[pUZ]};
-  const T w = sqrt(T(1.0) + W * W * s3quad(gi, u, u));
+  const T w = t_sqrt(T(1.0) + W * W * s3quad(gi, u, u));
   const T rho = pr[pRHO], P = pr[pP];
-  const T rh = rho * (T(1.0) + pr[pEPS] + P / rho);
+  const T rh = rho * (T(1.0) + pr[pEPS] + t_div(P, rho));
   E = rh * w * w - P;
   S[0] = rh * w * u[0]; S[1] = rh * w * u[1]; S[2] = rh * w * u[2];
-  const T iW2 = T(1.0) / (W * W);
+  const T iW2 = t_rcp(W * W);
   Sij[0] = rh * u[0] * u[0] + P * g.xx * iW2;
   Sij[1] = rh * u[0] * u[1] + P * g.xy * iW2;
   Sij[2] = rh * u[0] * u[2] + P * g.xz * iW2;
@@ -180,7 +180,7 @@ __device__ inline void z4c_source(const DevParams &p, const Z4cIn<T> &z, const G
   const T K = z.Kh + T(2.0) * z.Th;
   const T kap = pv<T>(p.kappa, p.fkappa) * fz;
   const T divb = z.db[0][0] + z.db[1][1] + z.db[2][2];
-  const T iW = T(1.0) / W;
+  const T iW = t_rcp(W);
 
   // physical D_i D_j alpha
   const T daW = s3quad(gi, z.dal, z.dW);
