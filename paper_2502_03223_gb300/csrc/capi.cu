@@ -795,8 +795,7 @@ void enqueue_sub_fill(Engine &e, Star &st, int l, int s, double theta) {
   const Lev &L = st.lv[l];
   const Lev &Pa = st.lv[l - 1];
   double *U = stage_state(st, l, s);
-  const long long np = (long long)Pa.px * Pa.pz;
-  run(e, K_TIME_INTERP, np * (NMET + NPRIM), [&] {
+  run(e, K_TIME_INTERP, (long long)time_interp_cells(Pa) * (NMET + NPRIM), [&] {
     launch_time_interp(Pa, st.uold[l - 1], st.pold[l - 1], st.pnow[l - 1], st.ut[l - 1], st.pt[l - 1], theta,
                        st.have_old[l - 1] ? 1 : 0, e.stream);
   });

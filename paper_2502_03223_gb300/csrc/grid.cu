@@ -399,12 +399,28 @@ void launch_b_rk_update(const Batch &b, const DevParams &p, int stage, double dt
 // (uold, pold), t^n (us, pnow), t^{n+1} (un, prim) in difference form about
 // t^n; first order through t^n, t^{n+1} for a primitive where
 // (p^{n+1} - p^n)(p^n - p^{n-1}) < 0, and everywhere while have_old = 0.
-// One thread per padded cell and plane (25 metric planes, then 6 primitives).
+// One thread per cell and plane (25 metric planes, then 6 primitives), on the
+// parent cells the child's buffer prolongation reads: child cells N + 1 ..
+// N + 8 lie in parent cells N/2 + 1 .. N/2 + 4, whose stencils reach from 4
+// below to 4 above, so the strip is {j >= N/2 - 3 or k >= N/2 - 3} of
+// [-3, N/2 + 8]^2.  (Over the whole padded plane it was memory-bound: 0.62 ms
+// per launch at 1024^2; the strip has 1/42 of those cells.)
 __global__ void k_time_interp(Lev P, const double *__restrict__ uold, const double *__restrict__ pold,
                               const double *__restrict__ pnow, double *__restrict__ ut, double *__restrict__ pt,
                               double theta, int have_old) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= P.px * P.pz) return;
+  int e = blockIdx.x * blockDim.x + threadIdx.x;
+  const int h = P.nx / 2, w = h + 12;        // strip columns [-3, h + 8]
+  int j, k;
+  if (e < 12 * w) {                          // rows h - 3 .. h + 8
+    j = -3 + e % w;
+    k = h - 3 + e / w;
+  } else {                                   // columns h - 3 .. h + 8 of the rows below
+    e -= 12 * w;
+    if (e >= 12 * h) return;
+    j = h - 3 + e % 12;
+    k = -3 + e / 12;
+  }
+  const int i = cid(P, j, k);
   const int f = blockIdx.y;
   const double wm = 0.5 * theta * (theta - 1.0), wp = 0.5 * theta * (theta + 1.0);
   if (f < NMET) {
@@ -419,9 +435,11 @@ __global__ void k_time_interp(Lev P, const double *__restrict__ uold, const doub
   }
 }
 
+int time_interp_cells(const Lev &P) { return 12 * (P.nx / 2 + 12) + 12 * (P.nx / 2); }
+
 void launch_time_interp(const Lev &P, const double *uold, const double *pold, const double *pnow, double *ut,
                         double *pt, double theta, int have_old, cudaStream_t s) {
-  const int n = P.px * P.pz;
+  const int n = time_interp_cells(P);
   k_time_interp<<<dim3((n + 255) / 256, NMET + NPRIM), 256, 0, s>>>(P, uold, pold, pnow, ut, pt, theta, have_old);
 }
 

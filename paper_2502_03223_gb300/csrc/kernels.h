@@ -145,6 +145,7 @@ void launch_rk_update(const Lev &L, const DevParams &p, double *Ust, int stage, 
                       cudaStream_t s);
 void launch_restrict(const Lev &C, const Lev &Pa, cudaStream_t s);
 // parent data at time t^n + theta (t^{n+1} - t^n) for a sub-cycled child (Sec. II.D)
+int time_interp_cells(const Lev &P);   // parent cells it interpolates
 void launch_time_interp(const Lev &P, const double *uold, const double *pold, const double *pnow, double *ut,
                         double *pt, double theta, int have_old, cudaStream_t s);
 void launch_reflux(const Lev &C, const Lev &Pa, double dt, cudaStream_t s);
