@@ -313,6 +313,14 @@ __device__ inline void enforce_algebraic(double m[NST], Sym3 *gi_out) {
 // RK stage combination on [1, jmax] x [1, kmax], then algebraic constraints
 // and primitive recovery.  Ust = stage state read (Un at stage 0, Us after);
 // the result is written to Us.
+// The stage update is bound by the latency of its ~100 loads per cell (30
+// fields of three registers), not by their bytes: with one field's loads at a
+// time and 160 registers (12 warps per SM) it moved 1.1 TB/s.  Groups of five
+// fields and 5 blocks per SM: 5.33 -> 4.13 ms per step of the migration star
+// (5 x 512^2), 0.58 -> 0.37 ms on the stable star (3 x 256^2); 3 and 4 blocks
+// 4.29 and 4.2, single fields at 4 blocks 4.77.
+constexpr int kRkGroup = 5, kRkBlocks = 5;
+static_assert(NMET % kRkGroup == 0 && NCONS % kRkGroup == 0, "the groups split at the conserved fields");
 template <bool SEED = false>
 __device__ __forceinline__ void rk_update_cell(const Lev &L, const DevParams &p, const double *__restrict__ Ust, int stage, double dt,
                                                    int jmax, int kmax, int j, int k, const MlpNet *net = nullptr) {
@@ -326,27 +334,46 @@ __device__ __forceinline__ void rk_update_cell(const Lev &L, const DevParams &p,
     const double x = (j - 0.5) * L.dx, z = (k - 0.5) * L.dz;
     held = x * x + z * z < p.r_hold2;
   }
-  for (int f = 0; f < NST; ++f) {
-    const size_t o = (size_t)f * P + id;
-    if (f < f0) { m[f] = L.us[o]; continue; }
-    if (f >= NMET && held) { m[f] = L.un[o]; continue; }
-    const double un = L.un[o], kk = L.rhs[o];
-    double out;
-    if (p.rk == SACRA_RK4) {
-      if (stage < 3) {
-        const double bw = stage == 0 ? 1.0 / 6.0 : 1.0 / 3.0;
-        L.ka[o] = (stage == 0 ? 0.0 : L.ka[o]) + bw * kk;
-        out = un + (stage == 2 ? 1.0 : 0.5) * dt * kk;
-      } else {
-        out = un + dt * (L.ka[o] + kk * (1.0 / 6.0));
-      }
-    } else {
-      if (stage == 0) out = un + dt * kk;
-      else if (stage == 1) out = 0.75 * un + 0.25 * Ust[o] + 0.25 * dt * kk;
-      else out = un * (1.0 / 3.0) + (2.0 / 3.0) * Ust[o] + (2.0 / 3.0) * dt * kk;
+  const bool rk4 = p.rk == SACRA_RK4;
+  // fields in groups: a group's loads are all in flight before the first is used
+#pragma unroll 1
+  for (int fb = f0; fb < NST; fb += kRkGroup) {
+    double un[kRkGroup], kk[kRkGroup], aux[kRkGroup];
+    const size_t ob = (size_t)fb * P + id;
+    const bool hold = held && fb >= NMET;          // the groups split at NMET
+    const double *pa = rk4 ? L.ka : Ust;           // the accumulator, or the stage state
+    const bool need_aux = stage > 0 && !hold;
+#pragma unroll
+    for (int i = 0; i < kRkGroup; ++i) {
+      const size_t o = ob + (size_t)i * P;
+      un[i] = L.un[o];
+      kk[i] = hold ? 0.0 : L.rhs[o];
+      aux[i] = need_aux ? pa[o] : 0.0;
     }
-    m[f] = out;
+#pragma unroll
+    for (int i = 0; i < kRkGroup; ++i) {
+      const size_t o = ob + (size_t)i * P;
+      double out;
+      if (hold) {
+        out = un[i];
+      } else if (rk4) {
+        if (stage < 3) {
+          const double bw = stage == 0 ? 1.0 / 6.0 : 1.0 / 3.0;
+          L.ka[o] = aux[i] + bw * kk[i];
+          out = un[i] + (stage == 2 ? 1.0 : 0.5) * dt * kk[i];
+        } else {
+          out = un[i] + dt * (aux[i] + kk[i] * (1.0 / 6.0));
+        }
+      } else {
+        if (stage == 0) out = un[i] + dt * kk[i];
+        else if (stage == 1) out = 0.75 * un[i] + 0.25 * aux[i] + 0.25 * dt * kk[i];
+        else out = un[i] * (1.0 / 3.0) + (2.0 / 3.0) * aux[i] + (2.0 / 3.0) * dt * kk[i];
+      }
+      m[fb + i] = out;
+    }
   }
+  if (f0)
+    for (int f = 0; f < f0; ++f) m[f] = L.us[(size_t)f * P + id];
   Sym3 gin;
   if (p.evolve) enforce_algebraic(m, &gin);
   if (held) {
@@ -369,7 +396,7 @@ __global__ void __launch_bounds__(128) k_rk_update(Lev L, DevParams p, const dou
 }
 
 template <bool SEED>
-__global__ void __launch_bounds__(128) kb_rk_update(Batch b, DevParams p, int stage, double dt) {
+__global__ void __launch_bounds__(128, SEED ? 2 : kRkBlocks) kb_rk_update(Batch b, DevParams p, int stage, double dt) {
   if constexpr (SEED) {
     // the learned recovery seed (one network for the batch) staged in shared memory
     __shared__ MlpNet snet;
