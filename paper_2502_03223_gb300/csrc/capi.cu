@@ -718,6 +718,7 @@ void enqueue_group_stage(Engine &e, int g, int s, double dt, bool reset_parent) 
     if (!kind_used(e, kind)) continue;
     const Batch b = batch_of(e, g, s, kind);
     run(e, kKindKid[kind], e.cells[plan_index(g, s, kind)], [&] { launch_kind(e, kind, b, s, dt); });
+    if (kind == B_POINT && !(e.dp.mixed & SACRA_MIXED_Z4C)) ++e.launches;   // two passes in FP64
   }
   if (s == e.S - 1) {
     if (g == 0 && e.lists) {

@@ -128,8 +128,6 @@ void launch_c2p_region(const Lev &L, const DevParams &p, double *U, int j0, int 
 void launch_cartoon(const Lev &L, const DevParams &p, const double *U, const double *tab, int tab_stride,
                     const double *tabw, cudaStream_t s);
 void launch_z4c_derivs(const Lev &L, const DevParams &p, const double *U, double *DS, int jmax, int kmax, cudaStream_t s);
-void launch_z4c_point(const Lev &L, const DevParams &p, const double *U, const double *DS, int jmax, int kmax,
-                      cudaStream_t s);
 int z4c_scratch_planes();
 int z4c_ricci_plane();
 

@@ -243,5 +243,130 @@ SF_HD double srsqrt(double a) {
   return pack61((u64)(rsqrt62(M, f) >> 1), 1023 - k, 0u);
 }
 
+// ---------------------------------------------------------------- block fixed point
+
+// A value of a group: (h 2^28 + l) 2^e, e the group's.  Loaded and normalised
+// values have |h| <= 2^28, |l| <= 2^28; sums of up to three of them are
+// formed limb by limb.
+struct Bf {
+  int h, l;
+};
+SF_HD Bf operator+(Bf a, Bf b) { return Bf{a.h + b.h, a.l + b.l}; }
+SF_HD Bf operator-(Bf a, Bf b) { return Bf{a.h - b.h, a.l - b.l}; }
+SF_HD Bf operator-(Bf a) { return Bf{-a.h, -a.l}; }
+SF_HD Bf twice(Bf a) { return Bf{2 * a.h, 2 * a.l}; }
+
+// Sum of products: H counts 2^56, C 2^28 units of 2^(ex + ey); the products
+// of the low limbs are left out (below 2^-56 of the largest possible product).
+// |h h'| <= 2^58 for one operand a sum of limbs, so 16 terms stay below 2^62.
+struct Acc {
+  i64 H = 0, C = 0;
+};
+SF_HD void mac(Acc &a, Bf x, Bf y) {
+  a.H += wide(x.h, y.h);
+  a.C += wide(x.h, y.l);
+  a.C += wide(x.l, y.h);
+}
+// the sum in units of 2^(ex + ey + kUnit)
+constexpr int kUnit = 56;
+SF_HD i64 fin(const Acc &a) { return a.H + (a.C >> 28); }
+
+SF_HD u64 shr_clamp(u64 u, int k) {              // u / 2^k, 0 for k >= 64
+#ifdef __CUDA_ARCH__
+  u64 r; asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(u), "r"(k)); return r;
+#else
+  return k < 64 ? u >> k : 0;
+#endif
+}
+SF_HD i64 sar_clamp(i64 u, int k) {
+#ifdef __CUDA_ARCH__
+  i64 r; asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(u), "r"(k)); return r;
+#else
+  return u >> (k < 63 ? k : 63);
+#endif
+}
+
+// x as a member of a group whose largest exponent field is E (E >= 64, so
+// that zeros and subnormals shift out): |h 2^28 + l| < 2^55, e = E - 1077
+SF_HD Bf conv(double x, int E) {
+  const i64 b = bits(x);
+  const unsigned hi = hiw(b), lo = low(b);
+  const int d = E - (int)((hi >> 20) & 0x7FFu);
+  const u64 u = ((u64)(((hi << 11) | (lo >> 21)) | 0x80000000u) << 32) | (lo << 11);
+  const u64 v = shr_clamp(u, 9 + d);
+  const int s = ((int)hi >> 31) | 1;
+  return Bf{(int)(v >> 28) * s, (int)((unsigned)v & 0xFFFFFFFu) * s};
+}
+SF_HD int field(double x) { return (int)(hiw(bits(x)) & 0x7FFFFFFFu); }   // exponent and top fraction bits
+SF_HD int imax(int a, int b) { return a > b ? a : b; }
+SF_HD int imin(int a, int b) { return a < b ? a : b; }
+
+template <int N>
+struct Grp {
+  Bf v[N];
+  int e;
+};
+
+// the group of N doubles; *top collects the largest exponent field seen
+// (2047: a value is not finite)
+template <int N>
+SF_HD void load(const double (&x)[N], Grp<N> &g, int &top) {
+  int m = 64 << 20;
+#pragma unroll
+  for (int i = 0; i < N; ++i) m = imax(m, field(x[i]));
+  const int E = m >> 20;
+  top = imax(top, E);
+#pragma unroll
+  for (int i = 0; i < N; ++i) g.v[i] = conv(x[i], E);
+  g.e = E - 1077;
+}
+
+// integers R (|R| < 2^62) in units of 2^eR as a group of 56-bit values
+template <int N>
+SF_HD void norm(const i64 (&R)[N], int eR, Grp<N> &g) {
+  u64 M = 1;
+#pragma unroll
+  for (int i = 0; i < N; ++i) M |= (u64)(R[i] ^ (R[i] >> 63));
+  const int n = clz64(M);                           // 1 .. 63
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const i64 w = (i64)((u64)R[i] << (n - 1));
+    g.v[i] = Bf{(int)(w >> 35), (int)((unsigned)(w >> 7) & 0xFFFFFFFu)};
+  }
+  g.e = eR + 8 - n;
+}
+
+// S 2^eS += T 2^eT, on the larger exponent's grid
+template <int N>
+SF_HD void align_add(i64 (&S)[N], int &eS, const i64 (&T)[N], int eT) {
+  const int e = imax(eS, eT), a = e - eS, b = e - eT;
+#pragma unroll
+  for (int i = 0; i < N; ++i) S[i] = sar_clamp(S[i], a) + sar_clamp(T[i], b);
+  eS = e;
+}
+
+// R 2^e as a double, rounded to nearest; results below the normal range are
+// zero, above it infinite
+SF_HD double to_double(i64 R, int e) {
+#if defined(__CUDA_ARCH__)
+  // one FP64 conversion, the exponent by an integer addition
+  const i64 b = bits((double)R);
+  const int er = (int)(hiw(b) >> 20) & 0x7FF;
+  if (er == 0) return 0.0;
+  if ((unsigned)(er + e - 1) >= 2045u) return er + e < 1 ? 0.0 : of_bits((b & (i64)(1ull << 63)) | 0x7FF0000000000000ll);
+  return of_bits(b + ((i64)e << 52));
+#else
+  const u64 s = (u64)(R >> 63);
+  const u64 a = ((u64)R ^ s) - s;
+  const int n = clz64(a);
+  const u64 u = a << (n & 63);
+  const int ex = 1086 - n + e;
+  const u64 m = (u >> 11) + ((u >> 10) & 1);        // 53 bits with the leading one (or the next power of two)
+  u64 b = m + ((u64)(unsigned)(ex - 1) << 52);
+  if ((unsigned)(ex - 1) >= 2045u || n == 64) b = (n == 64 || ex < 1) ? 0ull : 0x7FF0000000000000ull;
+  return of_bits((i64)(b | (s << 63)));
+#endif
+}
+
 }  // namespace sf
 }  // namespace sacra

@@ -10,6 +10,7 @@
 #include "kernels.h"
 #include "z4c.cuh"
 #include "fixed.cuh"
+#include "z4c_fx.cuh"
 
 namespace sacra {
 
@@ -935,20 +936,48 @@ __device__ __forceinline__ void z4c_point_cell(const Lev &L, const DevParams &p,
   for (int f = 0; f < NMET; ++f) L.rhs[(size_t)f * P + id] = to_f64<T>(src[f] + DS[(size_t)(DS_AK + f) * P + id]);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(128) k_z4c_point(Lev L, DevParams p, const double *__restrict__ U,
-                                                    const T *__restrict__ DS, int jmax, int kmax) {
-  z4c_point_cell<T>(L, p, U, DS, jmax, kmax, blockIdx.x * blockDim.x + threadIdx.x + 1, blockIdx.y * blockDim.y + threadIdx.y + 1);
+// cells the block fixed-point form hands back (non-finite values): out of
+// line, so that its registers do not weigh on the other path
+__device__ __noinline__ void z4c_point_fp64(const Lev &L, const DevParams &p, const double *__restrict__ U,
+                                            const double *__restrict__ DS, int jmax, int kmax, int j, int k,
+                                            double *__restrict__ rs_out) {
+  z4c_point_cell<double>(L, p, U, DS, jmax, kmax, j, k, rs_out);
+}
+
+// The FP64 right-hand side of a cell in block fixed point (z4c_fx.cuh), its
+// second pass handing cells back to the FP64 algebra.  Pass A's results wait
+// in the right-hand side's planes.
+__device__ __forceinline__ void z4c_cell_fx_a(const Lev &L, const double *__restrict__ U, const double *__restrict__ DS,
+                                              int jmax, int kmax, int j, int k) {
+  if (j > jmax || k > kmax) return;
+  const size_t P = L.P;
+  const int id = cid(L, j, k);
+  const double *u = U + id, *ds = DS + id;
+  double *r = L.rhs + id;
+  z4c_fx_a([&](int f) { return u[(size_t)f * P]; }, [&](int a, int q) { return ds[(size_t)(DS_D1 + 3 * a + q) * P]; },
+           [&](int f, double v) { r[(size_t)f * P] = v; });
+}
+
+__device__ __forceinline__ void z4c_cell_fx_b(const Lev &L, const DevParams &p, const double *__restrict__ U,
+                                              const double *__restrict__ DS, int jmax, int kmax, int j, int k,
+                                              double *__restrict__ rs_out) {
+  if (j > jmax || k > kmax) return;
+  const size_t P = L.P;
+  const int id = cid(L, j, k);
+  const double x = (j - 0.5) * L.dx, zc = (k - 0.5) * L.dz;
+  const double fz = exp(-t_div(x * x + zc * zc, p.r_z4 * p.r_z4));
+  const Z4cPar zp{p.kappa, p.eta_B, p.bssn};
+  const double *u = U + id, *ds = DS + id, *pr = L.prim + id;
+  double *r = L.rhs + id;
+  const bool ok = z4c_fx_b(
+      zp, [&](int f) { return u[(size_t)f * P]; }, [&](int a, int q) { return ds[(size_t)(DS_D1 + 3 * a + q) * P]; },
+      [&](int a, int q) { return ds[(size_t)(DS_D2 + 6 * a + q) * P]; }, [&](int f) { return ds[(size_t)(DS_AK + f) * P]; },
+      [&](int f) { return pr[(size_t)f * P]; }, [&](int f) { return r[(size_t)f * P]; }, fz,
+      [&](int f, double v) { r[(size_t)f * P] = v; }, rs_out ? rs_out + id : nullptr);
+  if (!ok) z4c_point_fp64(L, p, U, DS, jmax, kmax, j, k, rs_out);
 }
 
 // ---------------------------------------------------------------- host launchers
-
-void launch_z4c_point(const Lev &L, const DevParams &p, const double *U, const double *DS, int jmax, int kmax,
-                      cudaStream_t s) {
-  dim3 b(32, 4), g((jmax + 31) / 32, (kmax + 3) / 4);
-  if (p.mixed & SACRA_MIXED_Z4C) k_z4c_point<float><<<g, b, 0, s>>>(L, p, U, reinterpret_cast<const float *>(DS), jmax, kmax);
-  else k_z4c_point<double><<<g, b, 0, s>>>(L, p, U, DS, jmax, kmax);
-}
 
 void launch_cartoon(const Lev &L, const DevParams &p, const double *U, const double *tab, int tab_stride,
                     const double *tabw, cudaStream_t s) {
@@ -1001,12 +1030,28 @@ __global__ void __launch_bounds__(FDX * FDZ, 4) kb_z4c_derivs(Batch b, DevParams
   });
 }
 
-template <typename T>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 0) kb_z4c_point(Batch b, DevParams p, int store_rs) {
+// Pass A needs its 255 registers (3 blocks per SM: 40 % slower, spills), pass
+// B hides its loads better with four blocks per SM (7.3 ms per step of the
+// migration star for both passes, 7.4 with three, 8.0 with two).
+__global__ void __launch_bounds__(128, 2) kb_z4c_point_a(Batch b) {
+  for_tiles<false>(b, [&](const BL &q, const Tile &tl) {
+    z4c_cell_fx_a(q.L, q.U, reinterpret_cast<const double *>(q.DS), q.jmax, q.kmax, tl.j0 + threadIdx.x, tl.k0 + threadIdx.y);
+  });
+}
+
+__global__ void __launch_bounds__(128, 4) kb_z4c_point_b(Batch b, int store_rs) {
   for_tiles<false>(b, [&](const BL &q, const Tile &tl) {
     double *rs = store_rs ? reinterpret_cast<double *>(q.DS) + (size_t)DS_RS * q.L.P : nullptr;
-    z4c_point_cell<T>(q.L, q.P, q.U, reinterpret_cast<const T *>(q.DS), q.jmax, q.kmax, tl.j0 + threadIdx.x,
-                      tl.k0 + threadIdx.y, rs);
+    z4c_cell_fx_b(q.L, q.P, q.U, reinterpret_cast<const double *>(q.DS), q.jmax, q.kmax, tl.j0 + threadIdx.x,
+                  tl.k0 + threadIdx.y, rs);
+  });
+}
+
+__global__ void __launch_bounds__(128, 4) kb_z4c_point_f32(Batch b, int store_rs) {
+  for_tiles<false>(b, [&](const BL &q, const Tile &tl) {
+    double *rs = store_rs ? reinterpret_cast<double *>(q.DS) + (size_t)DS_RS * q.L.P : nullptr;
+    z4c_point_cell<float>(q.L, q.P, q.U, reinterpret_cast<const float *>(q.DS), q.jmax, q.kmax, tl.j0 + threadIdx.x,
+                          tl.k0 + threadIdx.y, rs);
   });
 }
 
@@ -1026,8 +1071,12 @@ void launch_b_z4c_derivs(const Batch &b, const DevParams &p, cudaStream_t s) {
 
 void launch_b_z4c_point(const Batch &b, const DevParams &p, cudaStream_t s, int store_rs) {
   if (b.ntiles <= 0) return;
-  if (p.mixed & SACRA_MIXED_Z4C) kb_z4c_point<float><<<b.grid, b.block, 0, s>>>(b, p, store_rs);
-  else kb_z4c_point<double><<<b.grid, b.block, 0, s>>>(b, p, store_rs);
+  if (p.mixed & SACRA_MIXED_Z4C) {
+    kb_z4c_point_f32<<<b.grid, b.block, 0, s>>>(b, store_rs);
+  } else {
+    kb_z4c_point_a<<<b.grid, b.block, 0, s>>>(b);
+    kb_z4c_point_b<<<b.grid, b.block, 0, s>>>(b, store_rs);
+  }
 }
 
 dim3 z4c_derivs_f32_block() { return dim3(DTX, DTZ); }
