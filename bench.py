@@ -501,7 +501,7 @@ def run_batch(args, dist, ws):
     brep = b.profile_report()
     b.profile(False)
     btot = sum(v[0] for v in brep.values())
-    per_level = ("k_parity_x", "k_parity_z", "k_outer", "k_prolong", "k_restrict", "k_reflux", "k_c2p_region",
+    per_level = ("k_parity", "k_outer", "k_prolong", "k_restrict", "k_reflux", "k_c2p_region",
                  "k_outflow", "k_time_interp")
     kshare = {k: round(v[0] / btot, 4) for k, v in sorted(brep.items(), key=lambda kv: -kv[1][0])}
     klaunch = {k: int(v[1]) for k, v in brep.items()}

@@ -118,10 +118,10 @@ bool compatible(const sacra_params *a, const sacra_params *b) {
 
 // kernel kinds for launch counting and the optional per-kernel profile
 enum Kid {
-  K_OUTFLOW, K_OUTER, K_PROLONG, K_PARITY_X, K_PARITY_Z, K_FLUX_X, K_FLUX_Z, K_HYDRO_DIV, K_CARTOON, K_Z4C_DERIVS,
+  K_OUTFLOW, K_OUTER, K_PROLONG, K_PARITY, K_FLUX_X, K_FLUX_Z, K_HYDRO_DIV, K_CARTOON, K_Z4C_DERIVS,
   K_Z4C_POINT, K_RK_UPDATE, K_RESTRICT, K_REFLUX, K_C2P, K_PRIM2CONS, K_DIAG, K_DIAG_FINAL, K_TIME_INTERP, K_COUNT
 };
-const char *kKidName[K_COUNT] = {"k_outflow", "k_outer", "k_prolong", "k_parity_x", "k_parity_z", "k_flux_x",
+const char *kKidName[K_COUNT] = {"k_outflow", "k_outer", "k_prolong", "k_parity", "k_flux_x",
                                  "k_flux_z", "k_hydro_rhs", "k_cartoon", "k_z4c_derivs", "k_z4c_point",
                                  "k_rk_update", "k_restrict", "k_reflux", "k_c2p_region", "k_prim2cons_all",
                                  "k_diag", "k_diag_final", "k_time_interp"};
@@ -482,7 +482,7 @@ void build_lists(Engine &e, std::vector<LItem> &items) {
           it.L = level_view(st, d, par);
           it.P = st.dp;
           it.B = s == 0 ? it.L.un : it.L.us;
-          add(Q, it, st.prm.nx, 8LL * (it.L.nz + GH));
+          add(Q, it, st.prm.nx, 8LL * (it.L.nz + GH) + 8LL * (it.L.nx + 2 * GH));
         }
       }
     open(e.l_oend[par]);
@@ -505,7 +505,7 @@ void build_lists(Engine &e, std::vector<LItem> &items) {
         it.L = level_view(st, d, par);
         it.P = st.dp;
         it.B = it.L.un;
-        add(Q, it, st.prm.nx, 8LL * (it.L.nz + GH));
+        add(Q, it, st.prm.nx, 8LL * (it.L.nz + GH) + 8LL * (it.L.nx + 2 * GH));
       }
       Engine::LList &R = e.l_restr[(size_t)par * D + d];
       open(R);
@@ -527,7 +527,7 @@ void build_lists(Engine &e, std::vector<LItem> &items) {
         it.L = level_view(st, l, par);
         it.P = st.dp;
         it.B = it.L.un;
-        add(e.l_ppar[par], it, st.prm.nx, 8LL * (it.L.nz + GH));
+        add(e.l_ppar[par], it, st.prm.nx, 8LL * (it.L.nz + GH) + 8LL * (it.L.nx + 2 * GH));
       }
   }
 }
@@ -598,8 +598,7 @@ void launch_kind(Engine &e, int kind, const Batch &b, int s, double dt) {
 
 void enqueue_parity(Engine &e, Star &st, int l, double *U) {
   const Lev &L = st.lv[l];
-  run(e, K_PARITY_X, 8LL * (L.nz + GH), [&] { launch_parity_x(L, U, e.stream); });
-  run(e, K_PARITY_Z, 8LL * (L.nx + 2 * GH), [&] { launch_parity_z(L, U, e.stream); });
+  run(e, K_PARITY, 8LL * (L.nz + GH) + 8LL * (L.nx + 2 * GH), [&] { launch_parity(L, U, e.stream); });
 }
 
 void enqueue_fill(Engine &e, Star &st, int s, double dt) {
@@ -630,8 +629,7 @@ void enqueue_fill(Engine &e, Star &st, int s, double dt) {
 void enqueue_parity_list(Engine &e, const Engine::LList &Q) {
   if (Q.n <= 0) return;
   const LItem *it = e.litems_dev + Q.off;
-  run(e, K_PARITY_X, Q.cells, [&] { launch_l_parity_x(it, Q.n, Q.max_nx, e.stream); });
-  run(e, K_PARITY_Z, Q.cells, [&] { launch_l_parity_z(it, Q.n, Q.max_nx, e.stream); });
+  run(e, K_PARITY, Q.cells, [&] { launch_l_parity(it, Q.n, Q.max_nx, e.stream); });
 }
 
 void enqueue_fill_lists(Engine &e, int s, double dt) {

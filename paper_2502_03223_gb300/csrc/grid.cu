@@ -30,42 +30,42 @@ __device__ __forceinline__ double sgn_z(int f) {
   }
 }
 
-// axis ghosts j in [-7, 0] for rows [1, nz+8]; blockIdx.z: plane (25 metric
-// fields, then the 6 primitives)
-__device__ __forceinline__ void parity_x_body(const Lev &L, double *__restrict__ U, int bx, int by, int f) {
-  const int j = -7 + (int)(bx * blockDim.x + threadIdx.x);
-  const int k = 1 + (int)(by * blockDim.y + threadIdx.y);
-  if (j > 0 || k > L.nz + GH) return;
-  const int d = cid(L, j, k), s = cid(L, 1 - j, k);
+// Axis and equator ghosts in one launch: columns [-7, 0] of rows [1, nz + 8]
+// and rows [-7, 0] of all columns [-7, nx + 8], indexed compactly (the rows
+// first).  A corner cell mirrors in both directions, from the cell 1 - j, 1 - k,
+// so no ghost is read.  by: plane (25 metric fields, then the 6 primitives).
+__host__ __device__ inline int parity_cells(int nx, int nz) { return GH * (nx + 2 * GH) + GH * (nz + GH); }
+
+__device__ __forceinline__ void parity_body(const Lev &L, double *__restrict__ U, int bx, int f) {
+  int e = (int)(bx * blockDim.x + threadIdx.x);
+  const int w = L.nx + 2 * GH;
+  int j, k;
+  if (e < GH * w) {
+    j = e % w - GH + 1;
+    k = e / w - GH + 1;
+  } else {
+    e -= GH * w;
+    if (e >= GH * (L.nz + GH)) return;
+    j = e % GH - GH + 1;
+    k = 1 + e / GH;
+  }
+  const int d = cid(L, j, k), s = cid(L, j <= 0 ? 1 - j : j, k <= 0 ? 1 - k : k);
+  double g = 1.0;
   if (f < NMET) {
+    if (j <= 0) g *= sgn_x(f);
+    if (k <= 0) g *= sgn_z(f);
     double *u = U + (size_t)f * L.P;
-    u[d] = sgn_x(f) * u[s];
+    u[d] = g * u[s];
   } else {
     const int q = f - NMET;
+    if (j <= 0 && (q == pUX || q == pUY)) g = -1.0;
+    if (k <= 0 && q == pUZ) g = -g;
     double *u = L.prim + (size_t)q * L.P;
-    u[d] = ((q == pUX || q == pUY) ? -1.0 : 1.0) * u[s];
+    u[d] = g * u[s];
   }
 }
 
-__global__ void k_parity_x(Lev L, double *__restrict__ U) { parity_x_body(L, U, blockIdx.x, blockIdx.y, blockIdx.z); }
-
-// equator ghosts k in [-7, 0] for all columns; blockIdx.z as above
-__device__ __forceinline__ void parity_z_body(const Lev &L, double *__restrict__ U, int bx, int by, int f) {
-  const int j = -7 + (int)(bx * blockDim.x + threadIdx.x);
-  const int k = -7 + (int)(by * blockDim.y + threadIdx.y);
-  if (j > L.nx + GH || k > 0) return;
-  const int d = cid(L, j, k), s = cid(L, j, 1 - k);
-  if (f < NMET) {
-    double *u = U + (size_t)f * L.P;
-    u[d] = sgn_z(f) * u[s];
-  } else {
-    const int q = f - NMET;
-    double *u = L.prim + (size_t)q * L.P;
-    u[d] = (q == pUZ ? -1.0 : 1.0) * u[s];
-  }
-}
-
-__global__ void k_parity_z(Lev L, double *__restrict__ U) { parity_z_body(L, U, blockIdx.x, blockIdx.y, blockIdx.z); }
+__global__ void __launch_bounds__(128) k_parity(Lev L, double *__restrict__ U) { parity_body(L, U, blockIdx.x, blockIdx.y); }
 
 // planar slab: zero-gradient copy into every ghost cell
 __global__ void k_outflow(Lev L, double *__restrict__ U) {
@@ -796,13 +796,9 @@ __global__ void k_diag_final(const double *__restrict__ partials, int n, double 
 // sized for the largest item; blocks beyond an item's extent do nothing.
 constexpr int kParityPlanes = NMET + NPRIM;
 
-__global__ void kl_parity_x(const LItem *__restrict__ items) {
-  const LItem &it = items[blockIdx.z / kParityPlanes];
-  parity_x_body(it.L, it.B, blockIdx.x, blockIdx.y, blockIdx.z % kParityPlanes);
-}
-__global__ void kl_parity_z(const LItem *__restrict__ items) {
-  const LItem &it = items[blockIdx.z / kParityPlanes];
-  parity_z_body(it.L, it.B, blockIdx.x, blockIdx.y, blockIdx.z % kParityPlanes);
+__global__ void __launch_bounds__(128) kl_parity(const LItem *__restrict__ items) {
+  const LItem &it = items[blockIdx.z];
+  parity_body(it.L, it.B, blockIdx.x, blockIdx.y);
 }
 __global__ void kl_outer(const LItem *__restrict__ items, double tau, int metric, int prims) {
   const LItem &it = items[blockIdx.z];
@@ -829,14 +825,9 @@ __global__ void kl_reflux(const LItem *__restrict__ items, double dt) {
   reflux_body(it.L, it.Pa, dt, blockIdx.x);
 }
 
-void launch_l_parity_x(const LItem *items, int n, int max_nx, cudaStream_t s) {
+void launch_l_parity(const LItem *items, int n, int max_nx, cudaStream_t s) {
   if (n <= 0) return;
-  kl_parity_x<<<dim3(1, (max_nx + GH + 15) / 16, n * kParityPlanes), dim3(8, 16), 0, s>>>(items);
-}
-
-void launch_l_parity_z(const LItem *items, int n, int max_nx, cudaStream_t s) {
-  if (n <= 0) return;
-  kl_parity_z<<<dim3((max_nx + 2 * GH + 31) / 32, 1, n * kParityPlanes), dim3(32, 8), 0, s>>>(items);
+  kl_parity<<<dim3((parity_cells(max_nx, max_nx) + 127) / 128, kParityPlanes, n), 128, 0, s>>>(items);
 }
 
 void launch_l_outer(const LItem *items, int n, int max_nx, double tau, int metric, int prims, cudaStream_t s) {
@@ -867,12 +858,8 @@ void launch_l_reflux(const LItem *items, int n, int max_nx, double dt, cudaStrea
 
 // ---------------------------------------------------------------- host launchers
 
-void launch_parity_x(const Lev &L, double *U, cudaStream_t s) {
-  k_parity_x<<<dim3(1, (L.nz + GH + 15) / 16, NMET + NPRIM), dim3(8, 16), 0, s>>>(L, U);
-}
-
-void launch_parity_z(const Lev &L, double *U, cudaStream_t s) {
-  k_parity_z<<<dim3((L.nx + 2 * GH + 31) / 32, 1, NMET + NPRIM), dim3(32, 8), 0, s>>>(L, U);
+void launch_parity(const Lev &L, double *U, cudaStream_t s) {
+  k_parity<<<dim3((parity_cells(L.nx, L.nz) + 127) / 128, NMET + NPRIM), 128, 0, s>>>(L, U);
 }
 
 void launch_outflow(const Lev &L, double *U, cudaStream_t s) {

@@ -90,8 +90,7 @@ struct LItem {
   const double *A;          // input state: the parent's stage state (prolongation), U^n (outer boundary)
   double *B;                // output state: the level's stage state (ghost fill), its U^n (restriction)
 };
-void launch_l_parity_x(const LItem *items, int n, int max_nx, cudaStream_t s);
-void launch_l_parity_z(const LItem *items, int n, int max_nx, cudaStream_t s);        // after the x parity
+void launch_l_parity(const LItem *items, int n, int max_nx, cudaStream_t s);
 void launch_l_outer(const LItem *items, int n, int max_nx, double tau, int metric, int prims, cudaStream_t s);
 void launch_l_prolong(const LItem *items, int n, int max_nx, int full, cudaStream_t s); // metric, then hydro
 void launch_l_restrict(const LItem *items, int n, int max_nx, cudaStream_t s);        // metric, then conserved
@@ -131,8 +130,7 @@ void launch_z4c_derivs(const Lev &L, const DevParams &p, const double *U, double
 int z4c_scratch_planes();
 int z4c_ricci_plane();
 
-void launch_parity_x(const Lev &L, double *U, cudaStream_t s);
-void launch_parity_z(const Lev &L, double *U, cudaStream_t s);
+void launch_parity(const Lev &L, double *U, cudaStream_t s);   // axis and equator ghosts
 void launch_outflow(const Lev &L, double *U, cudaStream_t s);
 void launch_outer(const Lev &L, const DevParams &p, const double *Un, double *U, double tau, cudaStream_t s);
 // two launches: the metric (one thread per buffer cell and field), then the hydro
