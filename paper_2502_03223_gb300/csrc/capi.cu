@@ -1384,7 +1384,6 @@ sacra_status read_state(Engine &e, int star, int level, int which, int field, do
   Lev &L = st.lv[level];
   const size_t np = (size_t)L.px * L.pz;
   const double *src = nullptr;
-  std::vector<double> tmp;
   if (which == SACRA_STATE_STEP || which == SACRA_STATE_STAGE || which == SACRA_RHS) {
     if (field < 0 || field >= NST) return fail(e, SACRA_ERR_ARG, "bad field");
     const double *base = which == SACRA_STATE_STEP ? L.un : (which == SACRA_STATE_STAGE ? L.us : L.rhs);
@@ -1395,22 +1394,20 @@ sacra_status read_state(Engine &e, int star, int level, int which, int field, do
   } else if (which != SACRA_STATUS) {
     return fail(e, SACRA_ERR_ARG, "unknown plane");
   }
-  tmp.resize(np);
+  const size_t ni = (size_t)L.nx * L.nz;
+  if (n != np && n != ni) return fail(e, SACRA_ERR_ARG, "n must be nx*nz or px*pz");
   if (which == SACRA_STATUS) {
     std::vector<int> sv(np);
     cudaMemcpyAsync(sv.data(), L.status, np * 4, cudaMemcpyDeviceToHost, e.stream);
     if (cudaStreamSynchronize(e.stream) != cudaSuccess) return cuda_check(e, "read_state");
-    for (size_t i = 0; i < np; ++i) tmp[i] = sv[i];
+    for (size_t i = 0; i < n; ++i)
+      host[i] = sv[n == np ? i : (size_t)cid(L, 1 + (int)(i % L.nx), 1 + (int)(i / L.nx))];
   } else {
-    cudaMemcpyAsync(tmp.data(), src, np * 8, cudaMemcpyDeviceToHost, e.stream);
+    // straight into the caller's buffer (no plane-sized host copy in between)
+    if (n == np) cudaMemcpyAsync(host, src, np * 8, cudaMemcpyDeviceToHost, e.stream);
+    else cudaMemcpy2DAsync(host, (size_t)L.nx * 8, src + cid(L, 1, 1), (size_t)L.px * 8, (size_t)L.nx * 8, L.nz,
+                           cudaMemcpyDeviceToHost, e.stream);
     if (cudaStreamSynchronize(e.stream) != cudaSuccess) return cuda_check(e, "read_state");
-  }
-  if (n == np) {
-    memcpy(host, tmp.data(), np * 8);
-  } else if (n == (size_t)L.nx * L.nz) {
-    for (int k = 1; k <= L.nz; ++k) memcpy(host + (size_t)(k - 1) * L.nx, tmp.data() + cid(L, 1, k), (size_t)L.nx * 8);
-  } else {
-    return fail(e, SACRA_ERR_ARG, "n must be nx*nz or px*pz");
   }
   return cuda_check(e, "read_state");
 }
