@@ -603,9 +603,35 @@ __device__ __forceinline__ float rn_add(float a, float b) { return __fadd_rn(a, 
 __device__ __forceinline__ float rn_sub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float rn_mul(float a, float b) { return __fmul_rn(a, b); }
 
+// In FP64 only the sums run on the FP64 pipe (a warp's comparison, minimum or
+// product there takes as long as an addition): signs, orders and minima are
+// taken on the bit patterns, doubling and halving on the exponent, with the
+// same values.  PPM took 175 of the 300 FP64 instructions of a face.
+__device__ __forceinline__ long long ordered(double v) {       // the order of doubles as that of integers
+  const long long b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFll);
+}
+
+// 2 min(|dl|, |dr|) and |t| / 2, the smaller with the sign of t, where dl and dr have one sign
+__device__ __forceinline__ double mc_slope_bits(double dl, double dr, double t) {
+  const long long kAbs = 0x7FFFFFFFFFFFFFFFll, kExp = 1ll << 52;
+  const long long bl = __double_as_longlong(dl), br = __double_as_longlong(dr), bt = __double_as_longlong(t);
+  const long long al = bl & kAbs, ar = br & kAbs, at = bt & kAbs;
+  if ((bl ^ br) < 0 || al == 0 || ar == 0) return 0.0;
+  const long long m = al < ar ? al : ar;
+  if (m < 2 * kExp || at < 2 * kExp) {                          // near the subnormal range
+    const double lim = fmin(fabs(0.5 * t), fmin(2.0 * fabs(dl), 2.0 * fabs(dr)));
+    return t > 0.0 ? lim : -lim;
+  }
+  const long long m2 = m + kExp, h = at - kExp;
+  const long long v = h < m2 ? h : m2;
+  return __longlong_as_double(v | (bt & ~kAbs));
+}
+
 template <typename T>
 __device__ inline T mc_slope(T am, T a0, T ap) {
   const T dl = rn_sub(a0, am), dr = rn_sub(ap, a0);
+  if constexpr (sizeof(T) == 8) return mc_slope_bits(dl, dr, rn_sub(ap, am));
   if (rn_mul(dl, dr) <= T(0)) return T(0);
   const T dc = rn_mul(T(0.5), rn_sub(ap, am));
   const T lim = fmin(fabs(dc), fmin(T(2) * fabs(dl), T(2) * fabs(dr)));
@@ -614,6 +640,24 @@ __device__ inline T mc_slope(T am, T a0, T ap) {
 
 template <typename T>
 __device__ inline void ppm_limit(T a0, T &aL, T &aR) {
+  if constexpr (sizeof(T) == 8) {
+    const long long oL = ordered(aL), o0 = ordered(a0), oR = ordered(aR);
+    const bool up = oL < o0 && o0 < oR, down = oL > o0 && o0 > oR;
+    if (!up && !down) {
+      aL = a0;
+      aR = a0;
+      return;
+    }
+    const double d = rn_sub(aR, aL);
+    const double a6 = rn_mul(6.0, __fma_rn(-0.5, rn_add(aL, aR), a0));
+    // d a6 > d^2 and -d^2 > d a6, divided by |d|
+    const long long b6 = __double_as_longlong(a6), bd = __double_as_longlong(d);
+    if ((b6 & 0x7FFFFFFFFFFFFFFFll) > (bd & 0x7FFFFFFFFFFFFFFFll)) {
+      if ((b6 ^ bd) >= 0) aL = rn_sub(rn_mul(3.0, a0), 2.0 * aR);
+      else aR = rn_sub(rn_mul(3.0, a0), 2.0 * aL);
+    }
+    return;
+  }
   if (rn_mul(rn_sub(aR, a0), rn_sub(a0, aL)) <= T(0)) {
     aL = a0;
     aR = a0;
@@ -629,6 +673,7 @@ __device__ inline void ppm_limit(T a0, T &aL, T &aR) {
 // interface value between cells a (slope sa) and b (slope sb), 4th order
 template <typename T>
 __device__ __forceinline__ T ppm_iface(T a, T b, T sa, T sb) {
+  if constexpr (sizeof(T) == 8) return __fma_rn(rn_sub(sb, sa), -1.0 / 6.0, __fma_rn(0.5, rn_sub(b, a), a));
   return rn_sub(rn_add(a, rn_mul(T(0.5), rn_sub(b, a))), rn_mul(rn_sub(sb, sa), T(1.0 / 6.0)));
 }
 

@@ -20,7 +20,7 @@ __device__ __forceinline__ double face6_fp64(const double *u, int s) {
 // fixed-point grid of their largest exponent (fixed.cuh; one guard bit, |v| <
 // 2^54, so the weighted sum, weight sum 356, stays below 2^63), one
 // conversion and an exact power-of-two scale: the interpolant rounded once,
-// in two FP64 operations instead of twelve.  Non-finite values and values
+// in one FP64 operation instead of twelve.  Non-finite values and values
 // near the bottom of the normal range take the FP64 form.
 __device__ __forceinline__ double face6(const double *u, int s) {
   long long b[6];
@@ -34,7 +34,14 @@ __device__ __forceinline__ double face6(const double *u, int s) {
 #pragma unroll
   for (int n = 0; n < 6; ++n) v[n] = fx::fix(b[n], E);
   const long long S = 3 * (v[0] + v[5]) - 25 * (v[1] + v[4]) + 150 * (v[2] + v[3]);
-  return (double)S * fx::unit(1.0 / 256.0, E);
+  // S 2^(E - kGrid - 8): one conversion, the exponent by an integer addition
+  // (|S| >= 2^-8 of the grid's largest value or 0, so the result stays normal
+  // for E >= 64 unless it cancels to fewer than the low bits)
+  const long long sb = fx::bits((double)S);
+  const int er = fx::expo(sb) + E - fx::kGrid - 8;
+  if (S == 0) return 0.0;
+  if (er < 1 || er > 2046) return ldexp((double)S, E - fx::kGrid - 8);
+  return __longlong_as_double(sb + ((long long)(E - fx::kGrid - 8) << 52));
 }
 
 // Face j+1/2 (dir 0, stride 1) or k+1/2 (dir 1, stride px) of cell (j, k):
