@@ -64,6 +64,27 @@ __device__ inline void flux_states_f64(const Lev &L, const DevParams &p, const d
     for (int v = 0; v < 5; ++v) pr[v] = L.prim[(size_t)pf[v] * P + id + s];
   const double alpha = face6(U + (size_t)fAL * P + id, s);
   const double W = face6(U + (size_t)fW * P + id, s);
+  // Equal states at rest (the atmosphere, most faces of a star's grid): the
+  // flux of that state, f - v_int q, in closed form.  With u_i = 0 only the
+  // pressure and the shift are left, and the tetrad's factors cancel:
+  // (D, E) -beta^n / W^3, normal momentum alpha P / W^3.
+  long long diff = 0;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) diff |= fx::bits(pl[v]) ^ fx::bits(pr[v]);
+#pragma unroll
+  for (int v = 1; v < 4; ++v) diff |= fx::bits(pl[v]) << 1;
+  if (diff == 0) {
+    const double bn = face6(U + (size_t)(DIR == 0 ? fBX : fBZ) * P + id, s);
+    const double iW = t_rcp(W), iW3 = iW * iW * iW;
+    const double rho = pl[0], pc = eos_pc(p, rho), Pp = p.adiabatic ? pc : pl[4];
+    const double a = -bn * iW3;
+    out[0] = a * rho;
+    out[4] = a * (rho * (1.0 + eos_ec(p, rho)) + (Pp - pc) * p.ith1);
+    out[1] = out[2] = out[3] = 0.0;
+    out[DIR == 0 ? 1 : 3] = alpha * iW3 * Pp;
+    *fb = 0;
+    return;
+  }
   double beta[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) beta[i] = face6(U + (size_t)(fBX + i) * P + id, s);
@@ -529,6 +550,32 @@ __device__ __forceinline__ void hydro_rhs_cell(const Lev &L, const DevParams &p,
   for (int f = 0; f < NPRIM; ++f) pr[f] = ld_as<T>(L.prim[(size_t)f * P + id]);
   const T rho = pr[pRHO], Pp = pr[pP];
   const T u[3] = {pr[pUX], pr[pUY], pr[pUZ]};
+  if constexpr (sizeof(T) == 8) {
+    if (DS != nullptr && !(p.mixed & SACRA_MIXED_Z4C) && u[0] == 0.0 && u[1] == 0.0 && u[2] == 0.0) {
+      // matter at rest (the atmosphere): only the pressure, its trace with
+      // K_ij = (At_ij + gt_ij K / 3) / W^2 and the gradients of alpha and W are left
+      const double *ds = reinterpret_cast<const double *>(DS) + id;
+      const double iW = t_rcp(W), iW3 = iW * iW * iW;
+      const double rh = rho * (1.0 + pr[pEPS]) + Pp;
+      const double trA = gi.xx * ld(fAXX) + gi.yy * ld(fAYY) + gi.zz * ld(fAZZ)
+                       + 2.0 * (gi.xy * ld(fAXY) + gi.xz * ld(fAXZ) + gi.yz * ld(fAYZ));
+      const double K = ld(fKH) + 2.0 * ld(fTH);
+      const double aP = al * Pp, c3 = -3.0 * aP * iW;
+      double s[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const double dal = ds[(size_t)(DS_D1 + 3 * d1_of(fAL) + 2 * e) * P], dW = ds[(size_t)(DS_D1 + 3 * d1_of(fW) + 2 * e) * P];
+        s[e] = iW3 * ((Pp - rh) * dal + c3 * dW);
+      }
+      double *rq = L.rhsq + id;
+      rq[0] = -div[0];
+      rq[P] = s[0] + (cyl ? t_div(aP * iW3, xd) : 0.0) - div[1];
+      rq[2 * P] = -div[2];
+      rq[3 * P] = s[1] - div[3];
+      rq[4 * P] = iW3 * aP * (trA + K) - div[4];
+      return;
+    }
+  }
   const T w = t_sqrt(T(1) + W * W * s3quad(gi, u, u));
   const T iw = t_rcp(w);
   const T rhw2 = rho * (T(1) + pr[pEPS] + t_div(Pp, rho)) * w * w;
