@@ -374,6 +374,25 @@ struct C2pD {
   double v, inv;
 };
 
+// signs and orders on the bit patterns: a comparison on the FP64 pipe takes as
+// long as an addition.  same_sign: x y > 0 for x, y that are not zero (false
+// for NaN, as the product's comparison is); less_pos: x < y for x, y >= 0;
+// less_any: x < y for any x (false for NaN) and any y but NaN
+__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+__device__ __forceinline__ bool is_finite(double x) { return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000; }
+__device__ __forceinline__ bool is_nan(double x) {
+  return (__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) > 0x7FF0000000000000ll;
+}
+__device__ __forceinline__ bool same_sign(double x, double y) {
+  return (__double2hiint(x) ^ __double2hiint(y)) >= 0 && !is_nan(x) && !is_nan(y);
+}
+__device__ __forceinline__ bool less_pos(double x, double y) { return __double_as_longlong(x) < __double_as_longlong(y); }
+__device__ __forceinline__ bool less_any(double x, double y) {
+  const long long a = __double_as_longlong(x), b = __double_as_longlong(y);
+  return (a ^ ((a >> 63) & 0x7FFFFFFFFFFFFFFFll)) < (b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFll)) && !(is_zero(x) && is_zero(y)) &&
+         !is_nan(x);
+}
+
 // Master functions of the recovery (Sec. II.C.4, Eq. c2p_fn); COLD selects
 // z - r / h_cold(rho(z)).  The thermal EOS sees eps clamped to the cold curve.
 // h = (1 + eps)(1 + a), a = P / (rho (1 + eps)), is formed as 1 + eps + P / rho.
@@ -381,16 +400,15 @@ template <bool COLD>
 __device__ inline double c2p_fun(const DevParams &p, double z, C2pD D, double qq, double r) {
   const double w2 = 1.0 + z * z, iw = t_rsqrt(w2);   // 1 / w: rho = D / w without a division
   const double w = w2 * iw;
-  const double rho = D.v * iw, irho = w * D.inv;
-  if (COLD) {
-    const double hc = 1.0 + eos_ec(p, rho) + eos_pc(p, rho) * irho;
-    return z - t_div(r, hc);
-  }
+  const double rho = D.v * iw;
+  const double ec = eos_ec(p, rho);
+  // P_cold / rho (K rho = eps_cold for one polytrope of Gamma = 2)
+  const double pr = p.gamma2 && p.n_pieces == 1 ? ec : eos_pc(p, rho) * (w * D.inv);
+  if (COLD) return z - t_div(r, 1.0 + ec + pr);
   double eps = w * qq - z * r + t_div(z * z, 1.0 + w);
-  const double emin = eos_ec(p, rho);
-  if (eps < emin) eps = emin;
-  const double P = eos_p(p, rho, eps);
-  return z - t_div(r, 1.0 + eps + P * irho);
+  if (less_any(eps, ec)) eps = ec;
+  // h = 1 + eps + P / rho, P / rho = P_cold / rho + (Gamma_th - 1)(eps - eps_cold)
+  return z - t_div(r, 1.0 + eps + (pr + (p.Gamma_th - 1.0) * (eps - ec)));
 }
 
 // Illinois bracketing iteration from the bracket [a, b] with the master
@@ -400,9 +418,9 @@ __device__ double illinois_from(const DevParams &p, double a, double fa, double 
                                 double r, int *its, int *ok) {
   *its = 0;
   *ok = 1;
-  if (fa == 0.0) return a;
-  if (fb == 0.0) return b;
-  if (fa * fb > 0.0) {
+  if (is_zero(fa)) return a;
+  if (is_zero(fb)) return b;
+  if (same_sign(fa, fb)) {
     *ok = 0;
     return fabs(fa) < fabs(fb) ? a : b;
   }
@@ -412,8 +430,8 @@ __device__ double illinois_from(const DevParams &p, double a, double fa, double 
     *its = it;
     c = t_div(a * fb - b * fa, fb - fa);
     const double fc = c2p_fun<COLD>(p, c, D, qq, r);
-    if (fc == 0.0) return c;
-    if (fc * fb > 0.0) {
+    if (is_zero(fc)) return c;
+    if (same_sign(fc, fb)) {
       b = c; fb = fc;
       if (last == -1) fa *= 0.5;
       last = -1;
@@ -422,7 +440,7 @@ __device__ double illinois_from(const DevParams &p, double a, double fa, double 
       if (last == +1) fb *= 0.5;
       last = +1;
     }
-    if (fabs(b - a) <= p.c2p_tol * fmax(fabs(c), 1e-30)) return c;
+    if (!less_any(p.c2p_tol * fmax(fabs(c), 1e-30), fabs(b - a))) return c;
   }
   *ok = 0;
   return c;
@@ -448,29 +466,39 @@ __device__ inline void atmosphere(const DevParams &p, double pr[NPRIM]) {
 // SEED: the learned seed is compiled in (and used when net is not null)
 template <bool SEED = false>
 __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W, const Sym3 &gt, double x,
-                                   double pr[NPRIM], const MlpNet *net = nullptr, const Sym3 *gi_known = nullptr) {
-  const Sym3 gi = gi_known ? *gi_known : s3inv(gt, (double *)nullptr);   // the caller may hold gt^-1
+                                   double pr[NPRIM], const MlpNet *net = nullptr, const Sym3 *gi_known = nullptr,
+                                   double gi_scale = 1.0) {
   const double W3 = W * W * W;
   const double D = q[0] * W3;
   double S[3] = {q[1] * W3, q[2] * W3, q[3] * W3};
   if (p.geometry == SACRA_CYLINDRICAL) S[1] = t_div(S[1], x);
   const double E = q[4] * W3;
-  if (!(D > 0.0) || !(E > 0.0) || !isfinite(D) || !isfinite(E) || !isfinite(S[0]) || !isfinite(S[1]) ||
-      !isfinite(S[2])) {
+  // D, E positive and finite, S_i finite
+  if ((unsigned)(__double2hiint(D) - 1) >= 0x7FEFFFFFu && !(D > 0.0 && is_finite(D)) ||
+      (unsigned)(__double2hiint(E) - 1) >= 0x7FEFFFFFu && !(E > 0.0 && is_finite(E)) ||
+      !is_finite(S[0]) || !is_finite(S[1]) || !is_finite(S[2])) {
     atmosphere(p, pr);
     prim_to_cons(p, pr, W, gt, x, q);
     return ST_ATM | ST_BAD;
   }
   // the recovery returns rho = D / w <= D (w >= 1, either branch), so D < rho_atm
   // ends in the atmosphere reset of Sec. II.C.4 whatever the solve gives: skip it
-  if (D < p.rho_atm) {
+  if (less_pos(D, p.rho_atm)) {
     atmosphere(p, pr);
     prim_to_cons(p, pr, W, gt, x, q);
     return ST_ATM;
   }
   int st = 0;
-  const double iD = t_rcp(D);
-  double r = t_div(t_sqrt(W * W * s3quad(gi, S, S)), D);
+  // the caller may hold gt^-1 (times a factor)
+  Sym3 gi = gi_known ? *gi_known : s3inv(gt, (double *)nullptr);
+  if (SEED && gi_known) {
+    gi.xx *= gi_scale; gi.xy *= gi_scale; gi.xz *= gi_scale;
+    gi.yy *= gi_scale; gi.yz *= gi_scale; gi.zz *= gi_scale;
+    gi_scale = 1.0;
+  }
+  // S_i = 0 (matter at rest): r = 0 without the contraction
+  double r = 0.0;
+  if (!is_zero(S[0]) || !is_zero(S[1]) || !is_zero(S[2])) r = t_div(t_sqrt(W * W * gi_scale * s3quad(gi, S, S)), D);
   if (p.adiabatic) {
     // "adiabatic" EOS (Sec. III): zero temperature, the energy equation is
     // discarded: the cold recovery from D and S_i alone, the Lorentz factor
@@ -482,7 +510,7 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
       st |= ST_KRESCALE;
     }
     int its, ok;
-    const double z = illinois<true>(p, 0.0, r, C2pD{D, iD}, 0.0, r, &its, &ok);
+    const double z = illinois<true>(p, 0.0, r, C2pD{D, t_rcp(D)}, 0.0, r, &its, &ok);
     if (!ok) st |= ST_NOCONV;
     const double iw = t_rsqrt(1.0 + z * z);
     const double rho = D * iw;
@@ -494,13 +522,38 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
     pr[pUX] = S[0] * iDh;
     pr[pUY] = S[1] * iDh;
     pr[pUZ] = S[2] * iDh;
-    if (rho < p.rho_atm) {
+    if (less_any(rho, p.rho_atm)) {
       atmosphere(p, pr);
       st |= ST_ATM;
     }
     prim_to_cons(p, pr, W, gt, x, q);
     return st;
   }
+  if (is_zero(r) && !p.mlp) {
+    // matter at rest: the bracket is z = 0, its master function vanishes there, w = 1
+    if (p.c2p_stats) {
+      atomicAdd(p.c2p_stats + 0, 2ull);
+      atomicAdd(p.c2p_stats + 3, 1ull);
+    }
+    double eps = sf::sdiv_rn(E, D) - 1.0, P;
+    const double ec = eos_ec(p, D);
+    if (less_any(eps, ec)) {
+      eps = ec;
+      P = eos_pc(p, D);
+      st |= ST_COLD;
+    } else {
+      P = eos_p(p, D, eps);
+    }
+    pr[pRHO] = D;
+    pr[pEPS] = eps;
+    pr[pP] = P;
+    pr[pUX] = S[0];
+    pr[pUY] = S[1];
+    pr[pUZ] = S[2];
+    if (st & ST_COLD) prim_to_cons(p, pr, W, gt, x, q);
+    return st;
+  }
+  const double iD = t_rcp(D);
   const C2pD Dd{D, iD};
   const double qq = sf::sdiv_rn(E, D) - 1.0;   // E / D - 1 is near the cold curve's eps: rounded as the division
   double k = t_div(r, 1.0 + qq);
@@ -512,13 +565,35 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
     k = kmax;
     st |= ST_KRESCALE;
   }
-  const double zlo = 0.5 * k * t_rsqrt(1.0 - 0.25 * k * k);
-  const double zhi = k * t_rsqrt(1.0 - k * k);
-  int its, ok;
+  int its = 0, ok = 1;
   double z = 0.0;
-  bool solved = false;
+  bool solved = false, slow = false;
   unsigned long long ev = 0, tried = 0, held = 0;
-  if (SEED && net && r > 0.0 && k >= net->kmin) {
+  if (r <= 1e-4 && qq >= 0.0 && p.c2p_maxit >= 8 && p.c2p_tol >= 1e-14) {
+    // Slow flow (most recoveries of a star's atmosphere): z = r / h(z) by two
+    // fixed-point steps from z = 0.  h varies by a few z^2 of itself, so the
+    // relative error is a few z^2 after the first step and some 30 z^4 < 1e-14
+    // after the second, below what the bracket is closed to (c2p_tol), with one
+    // evaluation instead of the bracket's two ends and three or more steps.
+    // The root lies in the bracket [k / 2, k] where h <= 2 (1 + q); else the
+    // iteration below says that there is no sign change.
+    const double ec = eos_ec(p, D);
+    const double e0 = less_any(qq, ec) ? ec : qq;
+    const double pr0 = p.gamma2 && p.n_pieces == 1 ? ec : eos_pc(p, D) * iD;
+    const double h0 = 1.0 + e0 + (pr0 + (p.Gamma_th - 1.0) * (e0 - ec));
+    if (h0 < 1.999 * (1.0 + qq)) {
+      z = t_div(r, h0);
+      z -= c2p_fun<false>(p, z, Dd, qq, r);
+      slow = solved = true;
+      ev = 2;
+    }
+  }
+  double zlo = 0.0, zhi = 0.0;
+  if (!solved) {
+    zlo = 0.5 * k * t_rsqrt(1.0 - 0.25 * k * k);
+    zhi = k * t_rsqrt(1.0 - k * k);
+  }
+  if (SEED && net && !solved && r > 0.0 && k >= net->kmin) {
     // learned seed: P / D -> v = r / (1 + q + P / D) -> z0 = v / sqrt(1 - v^2) (FP32).  The master
     // function at z0 tells the side of the root; the bracket is [z0, z0 (1 + delta)] or
     // [z0 (1 - delta), z0] inside [zlo, zhi], and the Illinois iteration itself is unchanged
@@ -565,9 +640,14 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
   double rho = t_div(D, w);
   double eps = w * qq - z * r + t_div(z * z, 1.0 + w);
   double P;
-  if (eps < eos_ec(p, rho)) {
-    z = illinois<true>(p, 0.0, r, Dd, qq, r, &its, &ok);
-    if (!ok) st |= ST_NOCONV;
+  if (less_any(eps, eos_ec(p, rho))) {
+    if (slow) {
+      z = t_div(r, 1.0 + eos_ec(p, D) + eos_pc(p, D) * iD);
+      z -= c2p_fun<true>(p, z, Dd, qq, r);
+    } else {
+      z = illinois<true>(p, 0.0, r, Dd, qq, r, &its, &ok);
+      if (!ok) st |= ST_NOCONV;
+    }
     w = t_sqrt(1.0 + z * z);
     rho = t_div(D, w);
     eps = eos_ec(p, rho);
@@ -583,7 +663,7 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
   pr[pUX] = S[0] * iDh;
   pr[pUY] = S[1] * iDh;
   pr[pUZ] = S[2] * iDh;
-  if (rho < p.rho_atm) {
+  if (less_any(rho, p.rho_atm)) {
     atmosphere(p, pr);
     st |= ST_ATM;
   }

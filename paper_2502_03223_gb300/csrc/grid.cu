@@ -286,105 +286,139 @@ __device__ __forceinline__ double t_rcbrt(double d) {
 
 // det gt = 1 and tr At = 0 after every stage (Sec. II.B.1):
 // gt <- d^(-1/3) gt, W <- d^(-1/6) W, At <- d^(-1/3)(At - gt tr/3), Khat += tr
-// gi_out: the inverse of the normalised conformal metric, gt^-1 / c13 with
-// 1 / c13 = det c13^2
-__device__ inline void enforce_algebraic(double m[NST], Sym3 *gi_out) {
-  Sym3 g;
-  g.xx = 1.0 + m[fHXX]; g.xy = m[fHXY]; g.xz = m[fHXZ]; g.yy = 1.0 + m[fHYY]; g.yz = m[fHYZ]; g.zz = 1.0 + m[fHZZ];
+// gi_out, s_out: the inverse of gt before and the factor 1 / c13 = det c13^2
+// that makes it the inverse of the normalised metric (the recovery applies it
+// to |S|^2, where it needs it)
+__device__ __forceinline__ void enforce_algebraic(double &W, double h[6], double A[6], double &Kh, Sym3 *gi_out,
+                                                  double *s_out) {
+  const Sym3 g{1.0 + h[0], h[1], h[2], 1.0 + h[3], h[4], 1.0 + h[5]};
   double det;
   const Sym3 gi = s3inv(g, &det);
-  const double tr = gi.xx * m[fAXX] + gi.yy * m[fAYY] + gi.zz * m[fAZZ]
-                  + 2.0 * (gi.xy * m[fAXY] + gi.xz * m[fAXZ] + gi.yz * m[fAYZ]);
+  const double tr = gi.xx * A[0] + gi.yy * A[3] + gi.zz * A[5] + 2.0 * (gi.xy * A[1] + gi.xz * A[2] + gi.yz * A[4]);
   const double c13 = t_rcbrt(det), c16 = t_sqrt(c13), tr3 = tr * (1.0 / 3.0);
   const double gv[6] = {g.xx, g.xy, g.xz, g.yy, g.yz, g.zz};
 #pragma unroll
   for (int a = 0; a < 6; ++a) {
-    m[fAXX + a] = c13 * (m[fAXX + a] - gv[a] * tr3);
-    const double gn = c13 * gv[a];
-    m[fHXX + a] = (a == 0 || a == 3 || a == 5) ? gn - 1.0 : gn;
+    A[a] = c13 * (A[a] - gv[a] * tr3);
+    h[a] = (a == 0 || a == 3 || a == 5) ? fma(c13, gv[a], -1.0) : c13 * gv[a];
   }
-  m[fW] *= c16;
-  m[fKH] += tr;
-  const double s = det * c13 * c13;
-  gi_out->xx = gi.xx * s; gi_out->xy = gi.xy * s; gi_out->xz = gi.xz * s;
-  gi_out->yy = gi.yy * s; gi_out->yz = gi.yz * s; gi_out->zz = gi.zz * s;
+  W *= c16;
+  Kh += tr;
+  *s_out = det * c13 * c13;
+  *gi_out = gi;
 }
 
 // RK stage combination on [1, jmax] x [1, kmax], then algebraic constraints
 // and primitive recovery.  Ust = stage state read (Un at stage 0, Us after);
 // the result is written to Us.
-// The stage update is bound by the latency of its ~100 loads per cell (30
-// fields of three registers), not by their bytes: with one field's loads at a
-// time and 160 registers (12 warps per SM) it moved 1.1 TB/s.  Groups of five
-// fields and 5 blocks per SM: 5.33 -> 4.13 ms per step of the migration star
-// (5 x 512^2), 0.58 -> 0.37 ms on the stable star (3 x 256^2); 3 and 4 blocks
-// 4.29 and 4.2, single fields at 4 blocks 4.77.
-constexpr int kRkGroup = 5, kRkBlocks = 5;
-static_assert(NMET % kRkGroup == 0 && NCONS % kRkGroup == 0, "the groups split at the conserved fields");
+//
+// The update is bound by the latency of its ~100 loads per cell (30 fields of
+// three registers) and by the FP64 pipe, not by its bytes.  The fields go
+// through in groups whose loads are all in flight together and whose indices
+// are compile-time constants, so that no field waits in local memory: the
+// eleven fields that are only combined, then those of the algebraic
+// constraints, then the conserved ones.  Five blocks per SM (four and six are
+// within 2 %).  With one field's loads at a time and three blocks per SM it
+// took 5.3 ms per step of the migration star (5 x 512^2), 4.1 with groups of
+// five fields through local memory, 2.9 now (with the recovery's closed forms
+// for matter at rest and slow flow, common.cuh); 42 -> 26 ms per coarse step
+// of 7 x 1024^2.
+constexpr int kRkBlocks = 5;
+struct RkTerm {
+  double un, kk, aux;
+};
 template <bool SEED = false>
 __device__ __forceinline__ void rk_update_cell(const Lev &L, const DevParams &p, const double *__restrict__ Ust, int stage, double dt,
                                                    int jmax, int kmax, int j, int k, const MlpNet *net = nullptr) {
   if (j > jmax || k > kmax) return;
   const size_t P = L.P;
   const int id = cid(L, j, k);
-  double m[NST];
-  const int f0 = p.evolve ? 0 : NMET;
   bool held = false;   // excised inner boundary: the hydro keeps U^n and is not recovered
   if (p.r_hold2 > 0.0) {
     const double x = (j - 0.5) * L.dx, z = (k - 0.5) * L.dz;
     held = x * x + z * z < p.r_hold2;
   }
   const bool rk4 = p.rk == SACRA_RK4;
-  // fields in groups: a group's loads are all in flight before the first is used
-#pragma unroll 1
-  for (int fb = f0; fb < NST; fb += kRkGroup) {
-    double un[kRkGroup], kk[kRkGroup], aux[kRkGroup];
-    const size_t ob = (size_t)fb * P + id;
-    const bool hold = held && fb >= NMET;          // the groups split at NMET
-    const double *pa = rk4 ? L.ka : Ust;           // the accumulator, or the stage state
-    const bool need_aux = stage > 0 && !hold;
-#pragma unroll
-    for (int i = 0; i < kRkGroup; ++i) {
-      const size_t o = ob + (size_t)i * P;
-      un[i] = L.un[o];
-      kk[i] = hold ? 0.0 : L.rhs[o];
-      aux[i] = need_aux ? pa[o] : 0.0;
-    }
-#pragma unroll
-    for (int i = 0; i < kRkGroup; ++i) {
-      const size_t o = ob + (size_t)i * P;
-      double out;
-      if (hold) {
-        out = un[i];
-      } else if (rk4) {
-        if (stage < 3) {
-          const double bw = stage == 0 ? 1.0 / 6.0 : 1.0 / 3.0;
-          L.ka[o] = aux[i] + bw * kk[i];
-          out = un[i] + (stage == 2 ? 1.0 : 0.5) * dt * kk[i];
-        } else {
-          out = un[i] + dt * (aux[i] + kk[i] * (1.0 / 6.0));
-        }
-      } else {
-        if (stage == 0) out = un[i] + dt * kk[i];
-        else if (stage == 1) out = 0.75 * un[i] + 0.25 * aux[i] + 0.25 * dt * kk[i];
-        else out = un[i] * (1.0 / 3.0) + (2.0 / 3.0) * aux[i] + (2.0 / 3.0) * dt * kk[i];
+  const double *pa = rk4 ? L.ka : Ust;             // the accumulator, or the stage state
+  const double bw = stage == 0 ? 1.0 / 6.0 : 1.0 / 3.0;
+  const double ck = (rk4 ? (stage == 2 ? 1.0 : 0.5) : (stage == 1 ? 0.25 : 2.0 / 3.0)) * dt;
+  auto load = [&](int f) {
+    const size_t o = (size_t)f * P + id;
+    return RkTerm{L.un[o], L.rhs[o], stage > 0 ? pa[o] : 0.0};
+  };
+  auto combine = [&](int f, const RkTerm &t) {
+    if (rk4) {
+      if (stage < 3) {
+        L.ka[(size_t)f * P + id] = t.aux + bw * t.kk;
+        return t.un + ck * t.kk;
       }
-      m[fb + i] = out;
+      return t.un + dt * (t.aux + t.kk * (1.0 / 6.0));
     }
-  }
-  if (f0)
-    for (int f = 0; f < f0; ++f) m[f] = L.us[(size_t)f * P + id];
+    if (stage == 0) return t.un + dt * t.kk;
+    if (stage == 1) return 0.75 * t.un + 0.25 * t.aux + ck * t.kk;
+    return t.un * (1.0 / 3.0) + (2.0 / 3.0) * t.aux + ck * t.kk;
+  };
+  double W, h[6];
   Sym3 gin;
-  if (p.evolve) enforce_algebraic(m, &gin);
+  double gis = 1.0;
+  if (p.evolve) {
+    constexpr int kFree[11] = {fGX, fGY, fGZ, fTH, fAL, fBX, fBY, fBZ, fBBX, fBBY, fBBZ};
+    {
+      RkTerm t[6];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) t[i] = load(kFree[i]);
+#pragma unroll
+      for (int i = 0; i < 6; ++i) L.us[(size_t)kFree[i] * P + id] = combine(kFree[i], t[i]);
+#pragma unroll
+      for (int i = 0; i < 5; ++i) t[i] = load(kFree[6 + i]);
+#pragma unroll
+      for (int i = 0; i < 5; ++i) L.us[(size_t)kFree[6 + i] * P + id] = combine(kFree[6 + i], t[i]);
+    }
+    double A[6], Kh;
+    {
+      RkTerm t[7];
+#pragma unroll
+      for (int i = 0; i < 7; ++i) t[i] = load(fW + i);            // W, h_ij
+      W = combine(fW, t[0]);
+#pragma unroll
+      for (int i = 0; i < 6; ++i) h[i] = combine(fHXX + i, t[1 + i]);
+#pragma unroll
+      for (int i = 0; i < 7; ++i) t[i] = load(fAXX + i);          // At_ij, Khat
+#pragma unroll
+      for (int i = 0; i < 6; ++i) A[i] = combine(fAXX + i, t[i]);
+      Kh = combine(fKH, t[6]);
+    }
+    enforce_algebraic(W, h, A, Kh, &gin, &gis);
+    L.us[(size_t)fW * P + id] = W;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      L.us[(size_t)(fHXX + i) * P + id] = h[i];
+      L.us[(size_t)(fAXX + i) * P + id] = A[i];
+    }
+    L.us[(size_t)fKH * P + id] = Kh;
+  } else {
+    W = L.us[(size_t)fW * P + id];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) h[i] = L.us[(size_t)(fHXX + i) * P + id];
+  }
+  double q[NCONS];
   if (held) {
-    for (int f = f0; f < NST; ++f) L.us[(size_t)f * P + id] = m[f];
+#pragma unroll
+    for (int v = 0; v < NCONS; ++v) L.us[(size_t)(fQD + v) * P + id] = L.un[(size_t)(fQD + v) * P + id];
     return;
   }
-  Sym3 g;
-  g.xx = 1.0 + m[fHXX]; g.xy = m[fHXY]; g.xz = m[fHXZ]; g.yy = 1.0 + m[fHYY]; g.yz = m[fHYZ]; g.zz = 1.0 + m[fHZZ];
+  {
+    RkTerm t[NCONS];
+#pragma unroll
+    for (int v = 0; v < NCONS; ++v) t[v] = load(fQD + v);
+#pragma unroll
+    for (int v = 0; v < NCONS; ++v) q[v] = combine(fQD + v, t[v]);
+  }
+  const Sym3 g{1.0 + h[0], h[1], h[2], 1.0 + h[3], h[4], 1.0 + h[5]};
   double pr[NPRIM];
-  const int st = cons_to_prim<SEED>(p, m + fQD, m[fW], g, (j - 0.5) * L.dx, pr, net, p.evolve ? &gin : nullptr);
-  for (int f = f0; f < NST; ++f) L.us[(size_t)f * P + id] = m[f];
+  const int st = cons_to_prim<SEED>(p, q, W, g, (j - 0.5) * L.dx, pr, net, p.evolve ? &gin : nullptr, gis);
+#pragma unroll
+  for (int v = 0; v < NCONS; ++v) L.us[(size_t)(fQD + v) * P + id] = q[v];
 #pragma unroll
   for (int f = 0; f < NPRIM; ++f) L.prim[(size_t)f * P + id] = pr[f];
   L.status[id] = st;

@@ -368,5 +368,64 @@ SF_HD double to_double(i64 R, int e) {
 #endif
 }
 
+// ---------------------------------------------------------------- the conformal metric
+
+// gt_ij = delta_ij + h_ij (order xx, xy, xz, yy, yz, zz); false where some
+// |h_ij| >= 2^21 (or is not finite)
+SF_HD bool metric_group(const double (&h)[6], Grp<6> &g) {
+  int m = 1023 << 20;
+#pragma unroll
+  for (int a = 0; a < 6; ++a) m = imax(m, field(h[a]));
+  const int E = m >> 20;
+  if (E > 1043) return false;
+#pragma unroll
+  for (int a = 0; a < 6; ++a) g.v[a] = conv(h[a], E);
+  g.e = E - 1077;
+  const int one = 1 << (26 - (E - 1023));
+  g.v[0].h += one; g.v[3].h += one; g.v[5].h += one;
+  return true;
+}
+
+// gt^ij as a group and as integers R in units of 2^eR; det gt in units of
+// 2^edet; false where det gt <= 0
+SF_HD bool metric_inverse(const Grp<6> &g, Grp<6> &gi, i64 (&R)[6], int &eR, i64 &det, int &edet) {
+  auto cof = [&](int a, int b, int c, int d) {     // g_a g_b - g_c g_d
+    Acc s;
+    mac(s, g.v[a], g.v[b]);
+    mac(s, -g.v[c], g.v[d]);
+    return fin(s);
+  };
+  R[0] = cof(3, 5, 4, 4);
+  R[1] = cof(2, 4, 1, 5);
+  R[2] = cof(1, 4, 2, 3);
+  R[3] = cof(0, 5, 2, 2);
+  R[4] = cof(1, 2, 0, 4);
+  R[5] = cof(0, 3, 1, 1);
+  Grp<6> c;
+  norm(R, 2 * g.e + kUnit, c);
+  Acc s;
+  mac(s, g.v[0], c.v[0]);
+  mac(s, g.v[1], c.v[1]);
+  mac(s, g.v[2], c.v[2]);
+  det = fin(s);
+  edet = g.e + c.e + kUnit;
+  if (det <= 0) return false;
+  const int n = clz64((u64)det);                   // det = m 2^(63 - n + edet), m in [1, 2)
+  const u64 u = (u64)det << n;
+  u64 M = (u >> 11) + ((u >> 10) & 1);
+  M = M >> 53 ? (1ull << 53) - 1 : M;
+  const i64 iv = rcp62((unsigned)(M >> 32), (unsigned)M) >> 7;   // at most 2^55
+  const Bf idet = Bf{(int)(iv >> 28), (int)((unsigned)iv & 0xFFFFFFFu)};
+#pragma unroll
+  for (int a = 0; a < 6; ++a) {
+    Acc q;
+    mac(q, c.v[a], idet);
+    R[a] = fin(q);
+  }
+  eR = c.e - 55 - (63 - n + edet) + kUnit;
+  norm(R, eR, gi);
+  return true;
+}
+
 }  // namespace sf
 }  // namespace sacra

@@ -75,52 +75,13 @@ SF_HD bool z4c_fx_a(FU U, F1 D1, FO put) {
   Grp<6> g, gi;
   double hd[6], gd[6];                              // h_ij, gt^ij
   {
-    int m = 1023 << 20;
 #pragma unroll
-    for (int a = 0; a < 6; ++a) { hd[a] = U(fHXX + a); m = imax(m, field(hd[a])); }
-    const int E = m >> 20;
-    if (E > 1043) { put(zOK, 0.0); return false; }
+    for (int a = 0; a < 6; ++a) hd[a] = U(fHXX + a);
+    i64 det, R[6];
+    int edet, eR;
+    if (!metric_group(hd, g) || !metric_inverse(g, gi, R, eR, det, edet)) { put(zOK, 0.0); return false; }
 #pragma unroll
-    for (int a = 0; a < 6; ++a) g.v[a] = conv(hd[a], E);
-    g.e = E - 1077;
-    const int one = 1 << (26 - (E - 1023));
-    g.v[0].h += one; g.v[3].h += one; g.v[5].h += one;
-    i64 R[6];
-    auto cof = [&](int a, int b, int c, int d) {   // g_a g_b - g_c g_d
-      Acc s;
-      mac(s, g.v[a], g.v[b]);
-      mac(s, -g.v[c], g.v[d]);
-      return fin(s);
-    };
-    R[0] = cof(3, 5, 4, 4);
-    R[1] = cof(2, 4, 1, 5);
-    R[2] = cof(1, 4, 2, 3);
-    R[3] = cof(0, 5, 2, 2);
-    R[4] = cof(1, 2, 0, 4);
-    R[5] = cof(0, 3, 1, 1);
-    Grp<6> c;
-    norm(R, 2 * g.e + kUnit, c);
-    Acc s;
-    mac(s, g.v[0], c.v[0]);
-    mac(s, g.v[1], c.v[1]);
-    mac(s, g.v[2], c.v[2]);
-    const i64 det = fin(s);
-    if (det <= 0) { put(zOK, 0.0); return false; }
-    const int n = clz64((u64)det);                 // det = m 2^(63 - n + e), m in [1, 2)
-    const u64 u = (u64)det << n;
-    u64 M = (u >> 11) + ((u >> 10) & 1);
-    M = M >> 53 ? (1ull << 53) - 1 : M;
-    const i64 iv = rcp62((unsigned)(M >> 32), (unsigned)M) >> 7;   // at most 2^55
-    const Bf idet = Bf{(int)(iv >> 28), (int)((unsigned)iv & 0xFFFFFFFu)};
-    const int eid = -55 - (63 - n + g.e + c.e + kUnit);
-#pragma unroll
-    for (int a = 0; a < 6; ++a) {
-      Acc q;
-      mac(q, c.v[a], idet);
-      R[a] = fin(q);
-      gd[a] = to_double(R[a], c.e + eid + kUnit);
-    }
-    norm(R, c.e + eid + kUnit, gi);
+    for (int a = 0; a < 6; ++a) gd[a] = to_double(R[a], eR);
   }
 #pragma unroll
   for (int a = 0; a < 6; ++a) put(zGI + a, gd[a]);
@@ -348,15 +309,9 @@ SF_HD bool z4c_fx_b(const Z4cPar &p, FU U, F1 D1, F2 D2, FA AK, FP PR, FS scr, d
   };
   Grp<6> g;
   {
-    int m = 1023 << 20;
 #pragma unroll
-    for (int a = 0; a < 6; ++a) { hd[a] = U(fHXX + a); m = imax(m, field(hd[a])); }
-    const int E = m >> 20;                          // at most 1043 (pass A)
-#pragma unroll
-    for (int a = 0; a < 6; ++a) g.v[a] = conv(hd[a], E);
-    g.e = E - 1077;
-    const int one = 1 << (26 - (E - 1023));
-    g.v[0].h += one; g.v[3].h += one; g.v[5].h += one;
+    for (int a = 0; a < 6; ++a) hd[a] = U(fHXX + a);
+    metric_group(hd, g);                            // in range: pass A
   }
   const double W = U(fW), al = U(fAL), iW = srcp(W), aW = al * iW, W2 = W * W;
   double Rc[6];                                     // gt_k(i d_j) Gt^k - gt^lm d_l d_m gt_ij / 2
