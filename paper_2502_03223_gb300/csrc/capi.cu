@@ -582,7 +582,8 @@ Batch batch_of(const Engine &e, int g, int s, int kind) {
   const Shape sh = kind_shape(e, kind);
   b.block = dim3(sh.x, sh.y);
   const long long nb = (long long)e.sms * e.cfg[kind].blocks_per_sm;
-  b.grid = (int)std::max(1LL, std::min<long long>(nb, b.ntiles));
+  b.parts = kind == B_DERIVS ? z4c_derivs_parts(e.dp, b.ntiles, e.sms) : 1;
+  b.grid = (int)std::max(1LL, std::min<long long>(nb, (long long)b.ntiles * b.parts));
   b.ctr = e.tctr + kind;
   return b;
 }
@@ -984,7 +985,8 @@ sacra_status tune(Engine &e, int reps) {
     bt.tiles = tune_tiles;
     bt.ntiles = (int)t.size();
     bt.block = dim3(sh.x, sh.y);
-    bt.grid = (int)std::max(1LL, std::min<long long>((long long)e.sms * m, bt.ntiles));
+    bt.parts = kind == B_DERIVS ? z4c_derivs_parts(e.dp, bt.ntiles, e.sms) : 1;
+    bt.grid = (int)std::max(1LL, std::min<long long>((long long)e.sms * m, (long long)bt.ntiles * bt.parts));
     bt.ctr = e.tctr + kind;
     zero_counters(e);
     launch_kind(e, kind, bt, 0, 0.0, e.stream);   // warm-up

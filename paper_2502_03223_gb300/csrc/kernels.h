@@ -27,7 +27,8 @@ struct BL {                 // one level of one star as a stage sees it
   double wbp;               // ... in the parent-boundary registers (wb dt_level / dt_parent)
 };
 struct Tile {               // one block's worth of cells of one level
-  int bl, j0, k0, pad;
+  int bl, j0, k0;
+  int part;                 // 0 in the list; set by a walk over parts (Batch::parts)
 };
 struct Batch {
   const BL *bl;             // device array
@@ -36,6 +37,7 @@ struct Batch {
   int grid;                 // persistent blocks
   dim3 block;               // tile shape = block shape
   int *ctr;                 // tiles handed out past the first gridDim.x (zero at the launch)
+  int parts = 1;            // every tile is walked once per part: all tiles of part 0, then of part 1, ...
 };
 // Walk over the tiles of a batched launch.  DYN: block b starts with tile b,
 // then takes the next tile not yet handed out from the launch's counter, so
@@ -53,8 +55,10 @@ __device__ __forceinline__ void for_tiles(const Batch &b, F &&f) {
   if constexpr (DYN) {
     __shared__ int next;
     int t = blockIdx.x;
-    while (t < b.ntiles) {
-      const Tile tl = b.tiles[t];
+    const int nt = b.ntiles * b.parts;
+    while (t < nt) {
+      Tile tl = b.tiles[t % b.ntiles];
+      tl.part = t / b.ntiles;
       const int *src = reinterpret_cast<const int *>(b.bl + tl.bl);
       int *dst = reinterpret_cast<int *>(&sb);
       for (int i = tid; i < (int)(sizeof(BL) / sizeof(int)); i += nth) dst[i] = src[i];
@@ -65,8 +69,9 @@ __device__ __forceinline__ void for_tiles(const Batch &b, F &&f) {
       t = next;
     }
   } else {
-    for (int t = blockIdx.x; t < b.ntiles; t += gridDim.x) {
-      const Tile tl = b.tiles[t];
+    for (int t = blockIdx.x; t < b.ntiles * b.parts; t += gridDim.x) {
+      Tile tl = b.tiles[t % b.ntiles];
+      tl.part = t / b.ntiles;
       const int *src = reinterpret_cast<const int *>(b.bl + tl.bl);
       int *dst = reinterpret_cast<int *>(&sb);
       for (int i = tid; i < (int)(sizeof(BL) / sizeof(int)); i += nth) dst[i] = src[i];
@@ -124,6 +129,8 @@ void launch_b_z4c_point(const Batch &b, const DevParams &p, cudaStream_t s, int 
 void launch_b_rk_update(const Batch &b, const DevParams &p, int stage, double dt, cudaStream_t s);
 // the derivative passes have fixed tile shapes (their shared-memory staging)
 dim3 z4c_derivs_f32_block();
+// parts (ranges of fields) in which a derivative pass walks its tiles
+int z4c_derivs_parts(const DevParams &p, int ntiles, int sms);
 dim3 z4c_derivs_f64_block();
 
 void launch_flux_x(const Lev &L, const DevParams &p, const double *U, int jmax, int kmax, double wb, int has_child,

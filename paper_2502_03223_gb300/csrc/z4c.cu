@@ -537,20 +537,30 @@ __device__ __forceinline__ T fdko(const double *u, int s) {
 // FP32; the cartoon planes it reads are FP32 as well.
 constexpr int DTX = 32, DTZ = 8, DHX = DTX + 8, DHZ = DTZ + 8;
 
-// calls fn(std::integral_constant<int, F>) for F = F0 .. NMET - 1 (compile-time field loop)
-template <int F0>
+// calls fn(std::integral_constant<int, F>) for F = F0 .. F1 - 1 (compile-time field loop)
+template <int F0, int F1>
 struct FieldLoop {
   template <class Fn>
   __device__ __forceinline__ static void run(Fn &&fn) {
-    fn(std::integral_constant<int, F0>{});
-    FieldLoop<F0 + 1>::run(fn);
+    if constexpr (F0 < F1) {
+      fn(std::integral_constant<int, F0>{});
+      FieldLoop<F0 + 1, F1>::run(fn);
+    }
   }
 };
-template <>
-struct FieldLoop<NMET> {
-  template <class Fn>
-  __device__ __forceinline__ static void run(Fn &&) {}
-};
+
+// The derivative passes walk their tiles in three parts, ranges of fields: W
+// and h_ij, then At_ij .. Theta, then alpha .. B^i (the fields of a part's
+// d_xy at the level edge, Eq. cartoon_bnd, are in that part).  A small grid
+// gets three times the blocks, each a third as long: a 3 x 48^2 star is one
+// wave of blocks that each ran through 25 fields, 84 -> 49 us per FP64 pass.
+// The FP32 pass, whose field loop is unrolled, keeps one part's code in the
+// instruction cache: 3.05 -> 2.38 ms per mixed step of the migration star
+// 5 x 512^2, 28.2 -> 20.4 ms per coarse step of 7 x 1024^2.  The FP64 pass
+// takes parts up to three waves of blocks (stable star 3 x 256^2: 0.83 ms
+// against 0.85); beyond, the parts' own set-up costs more than it gives
+// (migration star: 6.4 ms against 5.9).
+constexpr int kPart1 = fAXX, kPart2 = fAL, kParts = 3;   // the first fields of parts 1 and 2
 
 __host__ __device__ constexpr bool y_zero_c(int f) {
   return f == fW || f == fKH || f == fTH || f == fAL || f == fGZ || f == fBZ || f == fBBZ || f == fHZZ || f == fAZZ;
@@ -561,6 +571,7 @@ __host__ __device__ constexpr bool y_zero_c(int f) {
 // before field f's stencils run from the other buffer, and one barrier per
 // field separates a buffer's last reads from its next writes.
 constexpr int kStagePer = (DHX * DHZ + DTX * DTZ - 1) / (DTX * DTZ);   // staged points per thread and field
+template <int F0, int F1>
 __device__ __forceinline__ void z4c_derivs_f32_tile(const Lev &L, const DevParams &p, const double *__restrict__ U,
                                                     float *__restrict__ DS, int jmax, int kmax, int cyl, int j0, int k0,
                                                     float2 (*tiles)[DHZ][DHX]) {
@@ -606,14 +617,14 @@ __device__ __forceinline__ void z4c_derivs_f32_tile(const Lev &L, const DevParam
       }
     }
   };
-  fetch(0);
-  stage(tiles[0]);
+  fetch(F0);
+  stage(tiles[F0 & 1]);
   __syncthreads();
 
-  FieldLoop<0>::run([&](auto fc) {
+  FieldLoop<F0, F1>::run([&](auto fc) {
     constexpr int f = decltype(fc)::value;
     float2 (*tile)[DHX] = tiles[f & 1];
-    if constexpr (f + 1 < NMET) fetch(f + 1);
+    if constexpr (f + 1 < F1) fetch(f + 1);
     if (live) {
       const int cx = tx + 4, cz = tz + 4;
       const float2 c = tile[cz][cx];
@@ -680,7 +691,7 @@ __device__ __forceinline__ void z4c_derivs_f32_tile(const Lev &L, const DevParam
         ed[eq] = d1x;
       }
     }
-    if constexpr (f + 1 < NMET) stage(tiles[(f + 1) & 1]);
+    if constexpr (f + 1 < F1) stage(tiles[(f + 1) & 1]);
     __syncthreads();
   });
   if (live && edge) {
@@ -688,14 +699,18 @@ __device__ __forceinline__ void z4c_derivs_f32_tile(const Lev &L, const DevParam
     const float x = ((float)j - 0.5f) * L.f.dx;
     const float ix = 1.0f / x, ix2 = ix * ix;
     auto put = [&](int a, float v) { DS[(size_t)(DS_D2 + 6 * a + 1) * P + id] = v; };
-    put(8, ev[6] * ix2 - ed[6] * ix);
-    put(9, -ev[5] * ix2 + ed[5] * ix);
-    put(3, ev[4] * ix2 - ed[4] * ix);
-    put(5, -ev[2] * ix2 + ed[2] * ix);
-    const float txy = ev[1] * ix2 - ed[1] * ix;
-    put(1, 2.0f * txy);
-    put(4, -2.0f * txy);
-    put(2, (ev[3] - ev[0]) * ix2 + (ed[0] - ed[3]) * ix);
+    if constexpr (F0 <= fBX && fBZ < F1) {
+      put(8, ev[6] * ix2 - ed[6] * ix);
+      put(9, -ev[5] * ix2 + ed[5] * ix);
+    }
+    if constexpr (F0 <= fHXX && fHZZ < F1) {
+      put(3, ev[4] * ix2 - ed[4] * ix);
+      put(5, -ev[2] * ix2 + ed[2] * ix);
+      const float txy = ev[1] * ix2 - ed[1] * ix;
+      put(1, 2.0f * txy);
+      put(4, -2.0f * txy);
+      put(2, (ev[3] - ev[0]) * ix2 + (ed[0] - ed[3]) * ix);
+    }
   }
 }
 
@@ -731,7 +746,8 @@ template <typename T>
 __device__ __forceinline__ void z4c_derivs_cell(const Lev &L, const DevParams &p, const double *__restrict__ U,
                                                 double *__restrict__ DS, int jmax, int kmax, int cyl, int j, int k,
                                                 long long *sdn = nullptr, int *sde = nullptr, int j0 = 0,
-                                                long long (*tb)[FHZ][FHX] = nullptr, int k0 = 0) {
+                                                long long (*tb)[FHZ][FHX] = nullptr, int k0 = 0, int f0 = 0,
+                                                int f1 = NMET) {
   static_assert(sizeof(T) == 8, "the FP32 form is z4c_derivs_f32_tile");
   // Staged form (tb, sdn, sde given): the mixed derivative d_xz is the
   // x-difference of the z-difference numerators of the neighbouring columns,
@@ -788,17 +804,17 @@ __device__ __forceinline__ void z4c_derivs_cell(const Lev &L, const DevParams &p
     }
   };
   if (tb) {
-    fetch(0);
-    stage(tb[0]);
+    fetch(f0);
+    stage(tb[f0 & 1]);
     __syncthreads();
   }
 #pragma unroll 1
-  for (int f = 0; f < NMET; ++f) {
+  for (int f = f0; f < f1; ++f) {
     const int a1 = kD1Of[f], a2 = kD2Of[f];
     const bool yz = y_zero(f);
     const double *u = U + (size_t)f * P + id;
     long long (*tile)[FHX] = tb ? tb[f & 1] : nullptr;
-    if (tb && f + 1 < NMET) fetch(f + 1);
+    if (tb && f + 1 < f1) fetch(f + 1);
     long long cn = 0;                  // z-difference numerator of this thread's column ...
     int ce = 1;                        // ... on the grid 2^(ce - kGrid); -1: not finite
     if (active) {
@@ -996,7 +1012,7 @@ __device__ __forceinline__ void z4c_derivs_cell(const Lev &L, const DevParams &p
       if (active) DS[(size_t)(DS_D2 + 6 * a2 + 2) * P + id] = dxz;
     }
     if (tb) {
-      if (f + 1 < NMET) stage(tb[(f + 1) & 1]);
+      if (f + 1 < f1) stage(tb[(f + 1) & 1]);
       __syncthreads();
     }
   }
@@ -1008,14 +1024,18 @@ __device__ __forceinline__ void z4c_derivs_cell(const Lev &L, const DevParams &p
     auto val = [&](int f) { return U[(size_t)f * P + id]; };
     auto ddx = [&](int f) { return DS[(size_t)(DS_D1 + 3 * kD1Of[f]) * P + id]; };
     auto put = [&](int a, double v) { DS[(size_t)(DS_D2 + 6 * a + 1) * P + id] = v; };
-    put(8, val(fBY) * ix2 - ddx(fBY) * ix);
-    put(9, -val(fBX) * ix2 + ddx(fBX) * ix);
-    put(3, val(fHYZ) * ix2 - ddx(fHYZ) * ix);
-    put(5, -val(fHXZ) * ix2 + ddx(fHXZ) * ix);
-    const double txy = val(fHXY) * ix2 - ddx(fHXY) * ix;
-    put(1, 2.0 * txy);
-    put(4, -2.0 * txy);
-    put(2, (val(fHYY) - val(fHXX)) * ix2 + (ddx(fHXX) - ddx(fHYY)) * ix);
+    if (f0 <= fBX && fBZ < f1) {
+      put(8, val(fBY) * ix2 - ddx(fBY) * ix);
+      put(9, -val(fBX) * ix2 + ddx(fBX) * ix);
+    }
+    if (f0 <= fHXX && fHZZ < f1) {
+      put(3, val(fHYZ) * ix2 - ddx(fHYZ) * ix);
+      put(5, -val(fHXZ) * ix2 + ddx(fHXZ) * ix);
+      const double txy = val(fHXY) * ix2 - ddx(fHXY) * ix;
+      put(1, 2.0 * txy);
+      put(4, -2.0 * txy);
+      put(2, (val(fHYY) - val(fHXX)) * ix2 + (ddx(fHXX) - ddx(fHYY)) * ix);
+    }
   }
 }
 
@@ -1033,14 +1053,17 @@ __global__ void __launch_bounds__(128) k_z4c_derivs(Lev L, DevParams p, const do
 __global__ void __launch_bounds__(DTX * DTZ, 3) k_z4c_derivs_f32(Lev L, DevParams p, const double *__restrict__ U,
                                                               float *__restrict__ DS, int jmax, int kmax, int cyl) {
   __shared__ float2 tiles[2][DHZ][DHX];
-  z4c_derivs_f32_tile(L, p, U, DS, jmax, kmax, cyl, blockIdx.x * DTX + 1, blockIdx.y * DTZ + 1, tiles);
+  z4c_derivs_f32_tile<0, NMET>(L, p, U, DS, jmax, kmax, cyl, blockIdx.x * DTX + 1, blockIdx.y * DTZ + 1, tiles);
 }
 
 __global__ void __launch_bounds__(DTX * DTZ, 4) kb_z4c_derivs_f32(Batch b, DevParams p) {
   __shared__ float2 tiles[2][DHZ][DHX];
   const int cyl = p.geometry == SACRA_CYLINDRICAL;
   for_tiles<false>(b, [&](const BL &q, const Tile &tl) {
-    z4c_derivs_f32_tile(q.L, q.P, q.U, reinterpret_cast<float *>(q.DS), q.jmax, q.kmax, cyl, tl.j0, tl.k0, tiles);
+    float *ds = reinterpret_cast<float *>(q.DS);
+    if (tl.part == 0) z4c_derivs_f32_tile<0, kPart1>(q.L, q.P, q.U, ds, q.jmax, q.kmax, cyl, tl.j0, tl.k0, tiles);
+    else if (tl.part == 1) z4c_derivs_f32_tile<kPart1, kPart2>(q.L, q.P, q.U, ds, q.jmax, q.kmax, cyl, tl.j0, tl.k0, tiles);
+    else z4c_derivs_f32_tile<kPart2, NMET>(q.L, q.P, q.U, ds, q.jmax, q.kmax, cyl, tl.j0, tl.k0, tiles);
   });
 }
 
@@ -1217,7 +1240,9 @@ __global__ void __launch_bounds__(FDX * FDZ, 4) kb_z4c_derivs(Batch b, DevParams
   const int cyl = p.geometry == SACRA_CYLINDRICAL;
   for_tiles(b, [&](const BL &q, const Tile &tl) {
     z4c_derivs_cell<double>(q.L, q.P, q.U, reinterpret_cast<double *>(q.DS), q.jmax, q.kmax, cyl, tl.j0 + threadIdx.x,
-                            tl.k0 + threadIdx.y, sdn, sde, tl.j0, tb, tl.k0);
+                            tl.k0 + threadIdx.y, sdn, sde, tl.j0, tb, tl.k0,
+                            tl.part == 0 ? 0 : (tl.part == 1 ? kPart1 : kPart2),
+                            b.parts == 1 || tl.part == 2 ? NMET : (tl.part == 0 ? kPart1 : kPart2));
   });
 }
 
@@ -1270,6 +1295,10 @@ void launch_b_z4c_point(const Batch &b, const DevParams &p, cudaStream_t s, int 
   }
 }
 
+int z4c_derivs_parts(const DevParams &p, int ntiles, int sms) {
+  if (p.mixed & SACRA_MIXED_Z4C) return kParts;
+  return ntiles <= 12 * sms ? kParts : 1;           // three waves of the FP64 pass's four blocks per SM
+}
 dim3 z4c_derivs_f32_block() { return dim3(DTX, DTZ); }
 dim3 z4c_derivs_f64_block() { return dim3(FDX, FDZ); }
 
