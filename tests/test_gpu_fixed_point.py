@@ -75,3 +75,43 @@ def test_cells_outside_the_fixed_point_range(field, value):
     ok = np.isfinite(ref)
     scale = np.maximum(np.abs(ref), np.nanmax(np.where(ok, np.abs(ref), 0.0), axis=(1, 2), keepdims=True))
     assert np.all(np.abs(out[1] - ref)[ok] <= 1e-9 * scale[ok] + 1e-12)
+
+
+@pytest.mark.parametrize("eos", ["hybrid", "ideal", "pieces", "adiabatic"])
+def test_recovery_of_slow_matter(eos):
+    """The closed forms of the recovery (matter at rest, slow flow) and the iteration either side of
+    their threshold r = 1e-4, thermal and cold branch, against the oracle's iteration on the same
+    conserved state.  Bounds: the iteration closes its bracket to 1e-12 relative in z; eps comes from
+    E / D - 1 (rounded alike on both sides), so it carries a few 1e-16 absolute."""
+    kw = {"hybrid": dict(K=100.0, Gamma=2.0, Gamma_th=2.0), "ideal": dict(K=0.0, Gamma_th=5.0 / 3.0),
+          "pieces": dict(K=100.0, Gamma=2.0, Gamma_th=1.8, pwp=((1e-5, 2.4),)),
+          "adiabatic": dict(K=100.0, Gamma=2.0, Gamma_th=2.0, eos_adiabatic=1)}[eos]
+    cfg = dataclasses.replace(W.shock_tube_config(96, 40), rho_atm=1e-13, **kw)
+    rng = np.random.default_rng(11)
+    shape = (cfg.pz, cfg.px)
+    d = np.zeros((30,) + shape)
+    d[0] = d[18] = 1.0
+    rho = 10.0 ** rng.uniform(-8, -2, shape)
+    u = 10.0 ** rng.uniform(-14, -2, shape) * (rng.random(shape) > 0.1)       # a tenth at rest
+    phi = rng.uniform(0, 2 * np.pi, shape)
+    d[25] = rho
+    d[26], d[27], d[28] = u * np.cos(phi), 0.3 * u, u * np.sin(phi)
+    pc = W.cold_P(W.cold_pieces(cfg.K, cfg.Gamma, cfg.pwp), rho) if cfg.K else 1e-3 * rho
+    d[29] = pc * (1.0 + 10.0 ** rng.uniform(-2, 1, shape))
+    g = S.Sacra(cfg)
+    g.set_initial_data(0, S.PRIM_METRIC, d)
+    raw = g.read_level(0, np.zeros(30 * cfg.px * cfg.pz)).reshape(30, *shape)
+    if eos in ("hybrid", "pieces"):                                            # a third below the cold curve
+        cold = rng.random(shape) < 0.33
+        raw[29] = np.where(cold, raw[25] * (1.0 + 0.2 * (raw[29] / raw[25] - 1.0)), raw[29])
+    g.set_initial_data(0, S.RAW, raw)
+    o = O.Oracle(cfg)
+    o.set_level(0, 1, raw)
+    a = [g.read(0, S.PRIMS, f) for f in range(6)]
+    b = [o.read(0, 2, f) for f in range(6)]
+    assert np.array_equal(g.read(0, S.STATUS, 0).astype(int), o.read(0, 4, 0).astype(int))
+    for f in (1, 2, 3):
+        assert np.all(np.abs(a[f] - b[f]) <= 1e-11 * np.abs(b[f]) + 1e-300), (eos, f)
+    assert np.all(np.abs(a[0] - b[0]) <= 1e-14 * b[0])
+    assert np.all(np.abs(a[4] - b[4]) <= 1e-12 * b[4] + 1e-14 * b[0])
+    assert np.all(np.abs(a[5] - b[5]) <= 1e-12 * b[5] + 1e-14)
