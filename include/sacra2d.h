@@ -291,8 +291,8 @@ sacra_status sacra_set_tuning(sacra_ctx *c, int kind, int tile_x, int tile_y, in
    on DEVICE tuples (every fifth tuple, index % 5 == 4, is held out) with Adam
    for `steps` minibatches of batch_blocks x 128 tuples, lr decaying by a
    cosine to lr / 100; writes the packed network to DEVICE dev_net.  The
-   seed is tried only where k = r / (1 + q) >= kmin (slow flows, where the
-   plain bracket already converges in 2-3 evaluations, can skip it).
+   seed is tried only where k = r / (1 + q) >= kmin, and not in slow flow
+   (r <= 1e-4), which the recovery closes in two evaluations without a bracket.
    host_loss: NULL or `steps` floats (minibatch loss per step); host_report:
    NULL or 3 floats (held-out RMS error of log10(P / D), 99.9th percentile of
    the seed's relative z error, the bracket half-width delta chosen as four

@@ -67,18 +67,18 @@ __device__ __forceinline__ void parity_body(const Lev &L, double *__restrict__ U
 
 __global__ void __launch_bounds__(128) k_parity(Lev L, double *__restrict__ U) { parity_body(L, U, blockIdx.x, blockIdx.y); }
 
-// planar slab: zero-gradient copy into every ghost cell
+// planar slab: zero-gradient copy into every ghost cell; blockIdx.y: the plane
+// (30 state planes, then the 6 primitives; one plane after the other in a
+// thread took 13 us on a 400 x 4 slab)
 __global__ void k_outflow(Lev L, double *__restrict__ U) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= L.px * L.pz) return;
   const int j = i % L.px - GH + 1, k = i / L.px - GH + 1;
   if (j >= 1 && j <= L.nx && k >= 1 && k <= L.nz) return;
   const int jj = min(max(j, 1), L.nx), kk = min(max(k, 1), L.nz);
-  const int s = cid(L, jj, kk);
-  const size_t P = L.P;
-  for (int f = 0; f < NST; ++f) U[(size_t)f * P + i] = U[(size_t)f * P + s];
-#pragma unroll
-  for (int f = 0; f < NPRIM; ++f) L.prim[(size_t)f * P + i] = L.prim[(size_t)f * P + s];
+  const int f = (int)blockIdx.y;
+  double *u = f < NST ? U + (size_t)f * L.P : L.prim + (size_t)(f - NST) * L.P;
+  u[i] = u[cid(L, jj, kk)];
 }
 
 // Outer boundary of the coarsest level (Sec. II.B.3): Q = Q_inf + (1 - tau/r)
@@ -87,7 +87,7 @@ __global__ void k_outflow(Lev L, double *__restrict__ U) {
 // Threads: the L-shaped strip {j > nx or k > nz} of [1, nx+8] x [1, nz+8],
 // indexed compactly (rows k > nz first), times kOuterGroups groups of fields
 // (blockIdx.y) that share the interpolation weights.
-constexpr int kOuterGroups = 5;
+constexpr int kOuterGroups = 13;
 
 __device__ __forceinline__ void outer_body(const Lev &L, const double *__restrict__ Un, double *__restrict__ U,
                                            double tau, int metric, int prims, int bx, int group) {
@@ -617,13 +617,15 @@ __global__ void k_reflux(Lev C, Lev Pa, double dt) { reflux_body(C, Pa, dt, bloc
 // ---------------------------------------------------------------- diagnostics
 
 constexpr int DIAG_Q = 9;   // H^2 dV, Mx^2 dV, My^2 dV, Mz^2 dV, dV, qD dV, qSphi dV, rho_max, n_fail
-constexpr int DIAG_T = 128;
+constexpr int DIAG_T = 128;   // threads of the cells' kernel
+constexpr int DIAG_F = 1024;  // threads of the final sum, one block
 
 // Block reduction of the diagnostic sums (slot 7: maximum) in a fixed order, so
 // the result is the same on every run: a shuffle tree inside each warp, then
 // warp 0 combines the per-warp values the same way.  The block total ends in
 // acc of thread 0.
-__device__ __forceinline__ void diag_block_reduce(double acc[DIAG_Q], double (*sh)[DIAG_T / 32], int t) {
+template <int T>
+__device__ __forceinline__ void diag_block_reduce(double acc[DIAG_Q], double (*sh)[T / 32], int t) {
   const int lane = t & 31, w = t >> 5;
 #pragma unroll
   for (int q = 0; q < DIAG_Q; ++q) {
@@ -639,7 +641,7 @@ __device__ __forceinline__ void diag_block_reduce(double acc[DIAG_Q], double (*s
   if (w == 0) {
 #pragma unroll
     for (int q = 0; q < DIAG_Q; ++q) {
-      double v = lane < DIAG_T / 32 ? sh[q][lane] : (q == 7 ? -1e300 : 0.0);
+      double v = lane < T / 32 ? sh[q][lane] : (q == 7 ? -1e300 : 0.0);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         const double u = __shfl_down_sync(0xffffffffu, v, o);
@@ -800,24 +802,24 @@ __global__ void __launch_bounds__(DIAG_T) k_diag(Lev L, DevParams p, const S *__
       }
     }
   }
-  diag_block_reduce(acc, sh, t);
+  diag_block_reduce<DIAG_T>(acc, sh, t);
   if (t == 0)
 #pragma unroll
     for (int q = 0; q < DIAG_Q; ++q) partials[(size_t)blockIdx.x * DIAG_Q + q] = acc[q];
 }
 
 // fixed-order sum of the block partials (deterministic)
-__global__ void k_diag_final(const double *__restrict__ partials, int n, double *__restrict__ out) {
-  __shared__ double sh[DIAG_Q][DIAG_T / 32];
+__global__ void __launch_bounds__(DIAG_F) k_diag_final(const double *__restrict__ partials, int n, double *__restrict__ out) {
+  __shared__ double sh[DIAG_Q][DIAG_F / 32];
   const int t = threadIdx.x;
   double acc[DIAG_Q];
 #pragma unroll
   for (int q = 0; q < DIAG_Q; ++q) acc[q] = 0.0;
-  for (int b = t; b < n; b += DIAG_T)
+  for (int b = t; b < n; b += DIAG_F)
 #pragma unroll
     for (int q = 0; q < DIAG_Q; ++q)
       acc[q] = (q == 7) ? fmax(acc[q], partials[(size_t)b * DIAG_Q + q]) : acc[q] + partials[(size_t)b * DIAG_Q + q];
-  diag_block_reduce(acc, sh, t);
+  diag_block_reduce<DIAG_F>(acc, sh, t);
   if (t == 0)
 #pragma unroll
     for (int q = 0; q < DIAG_Q; ++q) out[q] = acc[q];
@@ -897,7 +899,7 @@ void launch_parity(const Lev &L, double *U, cudaStream_t s) {
 }
 
 void launch_outflow(const Lev &L, double *U, cudaStream_t s) {
-  k_outflow<<<(unsigned)((L.P + 255) / 256), 256, 0, s>>>(L, U);
+  k_outflow<<<dim3((unsigned)((L.P + 255) / 256), NST + NPRIM), 256, 0, s>>>(L, U);
 }
 
 void launch_outer(const Lev &L, const DevParams &p, const double *Un, double *U, double tau, cudaStream_t s) {
@@ -953,7 +955,7 @@ void launch_diag(const Lev &L, const DevParams &p, const double *DS, int covered
 }
 
 void launch_diag_final(const double *partials, int n, double *out, cudaStream_t s) {
-  k_diag_final<<<1, DIAG_T, 0, s>>>(partials, n, out);
+  k_diag_final<<<1, DIAG_F, 0, s>>>(partials, n, out);
 }
 
 }  // namespace sacra

@@ -550,11 +550,20 @@ __device__ __forceinline__ void hydro_rhs_cell(const Lev &L, const DevParams &p,
   for (int f = 0; f < NPRIM; ++f) pr[f] = ld_as<T>(L.prim[(size_t)f * P + id]);
   const T rho = pr[pRHO], Pp = pr[pP];
   const T u[3] = {pr[pUX], pr[pUY], pr[pUZ]};
+  // The sources take the first derivatives the stage's derivative pass has
+  // written when that pass ran in the same arithmetic (FP64 sources with the
+  // FP64 pass; FP32 sources with the FP32 pass, whose stencil sums of exact
+  // differences are the ones cd1 forms), else form their own
+  const bool use_ds = DS != nullptr && (sizeof(T) == 8) == !(p.mixed & SACRA_MIXED_Z4C);
+  // d_x (e = 0) or d_z (e = 1) of metric field f
+  auto d1 = [&](int f, int e) -> T {
+    if (use_ds) return reinterpret_cast<const T *>(DS)[(size_t)(DS_D1 + 3 * d1_of(f) + (e == 0 ? 0 : 2)) * P + id];
+    return cd1<T>(U + (size_t)f * P + id, st[e], i60[e]);
+  };
   if constexpr (sizeof(T) == 8) {
-    if (DS != nullptr && !(p.mixed & SACRA_MIXED_Z4C) && u[0] == 0.0 && u[1] == 0.0 && u[2] == 0.0) {
+    if (u[0] == 0.0 && u[1] == 0.0 && u[2] == 0.0) {
       // matter at rest (the atmosphere): only the pressure, its trace with
       // K_ij = (At_ij + gt_ij K / 3) / W^2 and the gradients of alpha and W are left
-      const double *ds = reinterpret_cast<const double *>(DS) + id;
       const double iW = t_rcp(W), iW3 = iW * iW * iW;
       const double rh = rho * (1.0 + pr[pEPS]) + Pp;
       const double trA = gi.xx * ld(fAXX) + gi.yy * ld(fAYY) + gi.zz * ld(fAZZ)
@@ -564,8 +573,7 @@ __device__ __forceinline__ void hydro_rhs_cell(const Lev &L, const DevParams &p,
       double s[2];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        const double dal = ds[(size_t)(DS_D1 + 3 * d1_of(fAL) + 2 * e) * P], dW = ds[(size_t)(DS_D1 + 3 * d1_of(fW) + 2 * e) * P];
-        s[e] = iW3 * ((Pp - rh) * dal + c3 * dW);
+        s[e] = iW3 * ((Pp - rh) * d1(fAL, e) + c3 * d1(fW, e));
       }
       double *rq = L.rhsq + id;
       rq[0] = -div[0];
@@ -588,16 +596,6 @@ __device__ __forceinline__ void hydro_rhs_cell(const Lev &L, const DevParams &p,
   // gt^ac v_c, used in v_a v_b d gt^ab = -(gt^ac v_c)(gt^bd v_d) d gt_cd
   T gv[3];
   s3vec(gi, vd, gv);
-  // The sources take the first derivatives the stage's derivative pass has
-  // written when that pass ran in the same arithmetic (FP64 sources with the
-  // FP64 pass; FP32 sources with the FP32 pass, whose stencil sums of exact
-  // differences are the ones cd1 forms), else form their own
-  const bool use_ds = DS != nullptr && (sizeof(T) == 8) == !(p.mixed & SACRA_MIXED_Z4C);
-  // d_x (e = 0) or d_z (e = 1) of metric field f
-  auto d1 = [&](int f, int e) -> T {
-    if (use_ds) return reinterpret_cast<const T *>(DS)[(size_t)(DS_D1 + 3 * d1_of(f) + (e == 0 ? 0 : 2)) * P + id];
-    return cd1<T>(U + (size_t)f * P + id, st[e], i60[e]);
-  };
   T src[2], dal[2];
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
