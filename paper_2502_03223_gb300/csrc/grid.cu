@@ -424,11 +424,6 @@ __device__ __forceinline__ void rk_update_cell(const Lev &L, const DevParams &p,
   L.status[id] = st;
 }
 
-__global__ void __launch_bounds__(128) k_rk_update(Lev L, DevParams p, const double *__restrict__ Ust, int stage, double dt,
-                                                   int jmax, int kmax) {
-  rk_update_cell(L, p, Ust, stage, dt, jmax, kmax, 1 + (int)(blockIdx.x * blockDim.x + threadIdx.x), 1 + (int)(blockIdx.y * blockDim.y + threadIdx.y));
-}
-
 template <bool SEED>
 __global__ void __launch_bounds__(128, SEED ? 2 : kRkBlocks) kb_rk_update(Batch b, DevParams p, int stage, double dt) {
   if constexpr (SEED) {
@@ -919,12 +914,6 @@ void launch_prolong(const Lev &L, const Lev &Pa, const DevParams &p, double *U, 
   const int n = prolong_cells(L, full);
   k_prolong_metric<<<dim3((n + 127) / 128, NMET), 128, 0, s>>>(L, Pa, U, Up, lo);
   k_prolong_hydro<<<(n + 127) / 128, 128, 0, s>>>(L, Pa, p, U, lo);
-}
-
-void launch_rk_update(const Lev &L, const DevParams &p, double *Ust, int stage, double dt, int jmax, int kmax,
-                      cudaStream_t s) {
-  dim3 b(32, 4), g((jmax + 31) / 32, (kmax + 3) / 4);
-  k_rk_update<<<g, b, 0, s>>>(L, p, Ust, stage, dt, jmax, kmax);
 }
 
 void launch_restrict(const Lev &C, const Lev &Pa, cudaStream_t s) {

@@ -155,8 +155,6 @@ void launch_outer(const Lev &L, const DevParams &p, const double *Un, double *U,
 void launch_prolong(const Lev &L, const Lev &Pa, const DevParams &p, double *U, const double *Up, int full,
                     cudaStream_t s);
 int prolong_cells(const Lev &L, int full);
-void launch_rk_update(const Lev &L, const DevParams &p, double *Ust, int stage, double dt, int jmax, int kmax,
-                      cudaStream_t s);
 void launch_restrict(const Lev &C, const Lev &Pa, cudaStream_t s);
 // parent data at time t^n + theta (t^{n+1} - t^n) for a sub-cycled child (Sec. II.D)
 int time_interp_cells(const Lev &P);   // parent cells it interpolates

@@ -489,45 +489,9 @@ __global__ void __launch_bounds__(128) k_cartoon_f32(Lev L, const double *__rest
 
 // ---------------------------------------------------------------- derivative pass
 
-// derivative scratch layout (planes): D1 first derivatives of the 16 fields
-// below (3 planes each), D2 second derivatives of 11 fields (6 planes each),
-// AK advection + KO of all 25 fields.
-__constant__ int kD1Fields[16] = {fW, fHXX, fHXY, fHXZ, fHYY, fHYZ, fHZZ, fKH, fGX, fGY, fGZ, fTH, fAL, fBX, fBY, fBZ};
-__constant__ int kD2Fields[11] = {fW, fHXX, fHXY, fHXZ, fHYY, fHYZ, fHZZ, fAL, fBX, fBY, fBZ};
-
 __device__ __forceinline__ bool y_zero(int f) {
   return f == fW || f == fKH || f == fTH || f == fAL || f == fGZ || f == fBZ || f == fBBZ || f == fHZZ || f == fAZZ;
 }
-
-// Stencils: the differences of the FP64 data are always taken in FP64; the
-// weighted sums run in arithmetic T (FP64, or FP32 in the mixed form).
-template <typename T>
-__device__ __forceinline__ T fd1(const double *u, int s, T idx) {
-  return (T(45) * T(u[s] - u[-s]) - T(9) * T(u[2 * s] - u[-2 * s]) + T(u[3 * s] - u[-3 * s])) * idx;
-}
-template <typename T>
-__device__ __forceinline__ T fd2(const double *u, int s, T idx2) {
-  const double u0 = u[0];
-  return (T(270) * (T(u[s] - u0) + T(u[-s] - u0)) - T(27) * (T(u[2 * s] - u0) + T(u[-2 * s] - u0))
-          + T(2) * (T(u[3 * s] - u0) + T(u[-3 * s] - u0))) * idx2;
-}
-// upwind-biased 6th-order derivative in the direction of the advecting velocity
-template <typename T>
-__device__ __forceinline__ T fdlop(const double *u, int s, T v, T idx) {
-  if (v == T(0)) return T(0);
-  const int t = v > T(0) ? s : -s;
-  const double u0 = u[0];
-  const T r = T(2) * T(u[-2 * t] - u0) - T(24) * T(u[-t] - u0) + T(80) * T(u[t] - u0) - T(30) * T(u[2 * t] - u0)
-            + T(8) * T(u[3 * t] - u0) - T(u[4 * t] - u0);
-  return (v > T(0) ? r : -r) * idx;
-}
-template <typename T>
-__device__ __forceinline__ T fdko(const double *u, int s) {
-  const double u0 = u[0];
-  return (T(u[4 * s] - u0) + T(u[-4 * s] - u0)) - T(8) * (T(u[3 * s] - u0) + T(u[-3 * s] - u0))
-       + T(28) * (T(u[2 * s] - u0) + T(u[-2 * s] - u0)) - T(56) * (T(u[s] - u0) + T(u[-s] - u0));
-}
-
 
 // Mixed-precision derivative pass.  The block stages each field's tile with
 // a 4-cell halo in shared memory as FP32 (hi, lo) splits (integer bit
