@@ -686,7 +686,8 @@ __device__ __forceinline__ float rn_mul(float a, float b) { return __fmul_rn(a, 
 // In FP64 only the sums run on the FP64 pipe (a warp's comparison, minimum or
 // product there takes as long as an addition): signs, orders and minima are
 // taken on the bit patterns, doubling and halving on the exponent, with the
-// same values.  PPM took 175 of the 300 FP64 instructions of a face.
+// same values: x- and z-faces 4.14 -> 3.65 ms each per step of the migration
+// star 5 x 512^2 (before the closed form of matter at rest).
 __device__ __forceinline__ long long ordered(double v) {       // the order of doubles as that of integers
   const long long b = __double_as_longlong(v);
   return b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFll);
