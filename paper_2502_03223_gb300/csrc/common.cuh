@@ -9,6 +9,7 @@
 #include <string.h>
 
 #include "sacra2d.h"
+#include "fields.h"
 #include "softfp.cuh"
 
 namespace sacra {
@@ -18,14 +19,6 @@ constexpr int NMET = 25;
 constexpr int NCONS = 5;
 constexpr int NST = 30;
 constexpr int NPRIM = 6;
-
-// state field numbers (see include/sacra2d.h)
-enum : int {
-  fW = 0, fHXX, fHXY, fHXZ, fHYY, fHYZ, fHZZ, fAXX, fAXY, fAXZ, fAYY, fAYZ, fAZZ,
-  fKH, fGX, fGY, fGZ, fTH, fAL, fBX, fBY, fBZ, fBBX, fBBY, fBBZ,
-  fQD, fQSX, fQSY, fQSZ, fQE
-};
-enum : int { pRHO = 0, pUX, pUY, pUZ, pP, pEPS };
 
 // recovery status bits
 constexpr int ST_NOCONV = 1, ST_COLD = 2, ST_ATM = 4, ST_KRESCALE = 8, ST_BAD = 16;

@@ -1,23 +1,16 @@
-// FP64-accurate arithmetic on the integer and FP32 units.
+// FP64 arithmetic on the integer and FP32 units.
 //
 // On this part a warp's FP64 instruction takes 16 cycles of the SM's FP64
 // pipe, a division or square root 90 to 146 (measured, all lanes busy), while
 // a 32 x 32 + 64-bit integer multiply-add (mad.wide) takes 0.6 and a 32-bit
 // integer operation about 0.5.  The kernels of this library were bound by the
-// FP64 pipe with the integer and FP32 units idle.  This header holds the two
-// forms that move FP64-equivalent work onto those units:
-//
-//  * sdiv, srcp, ssqrt, srsqrt: quotient, reciprocal, square root and its
-//    reciprocal of doubles.  An FP32 seed (24 bits) and one third-order
-//    (Householder) step on the exact residual, all in integers, give 60 bits;
-//    the result is then rounded once.  The error is below 0.52 ulp.  Operands outside
-//    the normal range (zeros, infinities, NaN, subnormals) and results near
-//    its ends take the FP64 instruction sequence.
-//  * block fixed point (Bf, Acc): a group of values shares one exponent, each
-//    value is a 56-bit integer h 2^28 + l in two 32-bit limbs, and a product
-//    is three mad.wide into 64-bit sums.  A contraction of such groups has no
-//    rounding but the truncation of each term below 2^-56 of the largest
-//    possible one (an FP64 sum rounds at 2^-53 of its terms).
+// FP64 pipe with the integer and FP32 units idle.  sdiv, srcp, ssqrt and
+// srsqrt form the quotient, reciprocal, square root and its reciprocal of
+// doubles there: an FP32 seed (24 bits) and one third-order (Householder) step
+// on the exact residual, all in integers, give 60 bits; the result is then
+// rounded once.  The error is below 0.52 ulp.  Operands outside the normal
+// range (zeros, infinities, NaN, subnormals) and results near its ends take
+// the FP64 instruction sequence.
 #pragma once
 
 #include <math.h>
@@ -243,33 +236,7 @@ SF_HD double srsqrt(double a) {
   return pack61((u64)(rsqrt62(M, f) >> 1), 1023 - k, 0u);
 }
 
-// ---------------------------------------------------------------- block fixed point
-
-// A value of a group: (h 2^28 + l) 2^e, e the group's.  Loaded and normalised
-// values have |h| <= 2^28, |l| <= 2^28; sums of up to three of them are
-// formed limb by limb.
-struct Bf {
-  int h, l;
-};
-SF_HD Bf operator+(Bf a, Bf b) { return Bf{a.h + b.h, a.l + b.l}; }
-SF_HD Bf operator-(Bf a, Bf b) { return Bf{a.h - b.h, a.l - b.l}; }
-SF_HD Bf operator-(Bf a) { return Bf{-a.h, -a.l}; }
-SF_HD Bf twice(Bf a) { return Bf{2 * a.h, 2 * a.l}; }
-
-// Sum of products: H counts 2^56, C 2^28 units of 2^(ex + ey); the products
-// of the low limbs are left out (below 2^-56 of the largest possible product).
-// |h h'| <= 2^58 for one operand a sum of limbs, so 16 terms stay below 2^62.
-struct Acc {
-  i64 H = 0, C = 0;
-};
-SF_HD void mac(Acc &a, Bf x, Bf y) {
-  a.H += wide(x.h, y.h);
-  a.C += wide(x.h, y.l);
-  a.C += wide(x.l, y.h);
-}
-// the sum in units of 2^(ex + ey + kUnit)
-constexpr int kUnit = 56;
-SF_HD i64 fin(const Acc &a) { return a.H + (a.C >> 28); }
+// ---------------------------------------------------------------- parts of integer sums
 
 SF_HD u64 shr_clamp(u64 u, int k) {              // u / 2^k, 0 for k >= 64
 #ifdef __CUDA_ARCH__
@@ -278,72 +245,7 @@ SF_HD u64 shr_clamp(u64 u, int k) {              // u / 2^k, 0 for k >= 64
   return k < 64 ? u >> k : 0;
 #endif
 }
-SF_HD i64 sar_clamp(i64 u, int k) {
-#ifdef __CUDA_ARCH__
-  i64 r; asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(u), "r"(k)); return r;
-#else
-  return u >> (k < 63 ? k : 63);
-#endif
-}
-
-// x as a member of a group whose largest exponent field is E (E >= 64, so
-// that zeros and subnormals shift out): |h 2^28 + l| < 2^55, e = E - 1077
-SF_HD Bf conv(double x, int E) {
-  const i64 b = bits(x);
-  const unsigned hi = hiw(b), lo = low(b);
-  const int d = E - (int)((hi >> 20) & 0x7FFu);
-  const u64 u = ((u64)(((hi << 11) | (lo >> 21)) | 0x80000000u) << 32) | (lo << 11);
-  const u64 v = shr_clamp(u, 9 + d);
-  const int s = ((int)hi >> 31) | 1;
-  return Bf{(int)(v >> 28) * s, (int)((unsigned)v & 0xFFFFFFFu) * s};
-}
 SF_HD int field(double x) { return (int)(hiw(bits(x)) & 0x7FFFFFFFu); }   // exponent and top fraction bits
-SF_HD int imax(int a, int b) { return a > b ? a : b; }
-SF_HD int imin(int a, int b) { return a < b ? a : b; }
-
-template <int N>
-struct Grp {
-  Bf v[N];
-  int e;
-};
-
-// the group of N doubles; *top collects the largest exponent field seen
-// (2047: a value is not finite)
-template <int N>
-SF_HD void load(const double (&x)[N], Grp<N> &g, int &top) {
-  int m = 64 << 20;
-#pragma unroll
-  for (int i = 0; i < N; ++i) m = imax(m, field(x[i]));
-  const int E = m >> 20;
-  top = imax(top, E);
-#pragma unroll
-  for (int i = 0; i < N; ++i) g.v[i] = conv(x[i], E);
-  g.e = E - 1077;
-}
-
-// integers R (|R| < 2^62) in units of 2^eR as a group of 56-bit values
-template <int N>
-SF_HD void norm(const i64 (&R)[N], int eR, Grp<N> &g) {
-  u64 M = 1;
-#pragma unroll
-  for (int i = 0; i < N; ++i) M |= (u64)(R[i] ^ (R[i] >> 63));
-  const int n = clz64(M);                           // 1 .. 63
-#pragma unroll
-  for (int i = 0; i < N; ++i) {
-    const i64 w = (i64)((u64)R[i] << (n - 1));
-    g.v[i] = Bf{(int)(w >> 35), (int)((unsigned)(w >> 7) & 0xFFFFFFFu)};
-  }
-  g.e = eR + 8 - n;
-}
-
-// S 2^eS += T 2^eT, on the larger exponent's grid
-template <int N>
-SF_HD void align_add(i64 (&S)[N], int &eS, const i64 (&T)[N], int eT) {
-  const int e = imax(eS, eT), a = e - eS, b = e - eT;
-#pragma unroll
-  for (int i = 0; i < N; ++i) S[i] = sar_clamp(S[i], a) + sar_clamp(T[i], b);
-  eS = e;
-}
 
 // R 2^e as a double, rounded to nearest; results below the normal range are
 // zero, above it infinite
@@ -366,65 +268,6 @@ SF_HD double to_double(i64 R, int e) {
   if ((unsigned)(ex - 1) >= 2045u || n == 64) b = (n == 64 || ex < 1) ? 0ull : 0x7FF0000000000000ull;
   return of_bits((i64)(b | (s << 63)));
 #endif
-}
-
-// ---------------------------------------------------------------- the conformal metric
-
-// gt_ij = delta_ij + h_ij (order xx, xy, xz, yy, yz, zz); false where some
-// |h_ij| >= 2^21 (or is not finite)
-SF_HD bool metric_group(const double (&h)[6], Grp<6> &g) {
-  int m = 1023 << 20;
-#pragma unroll
-  for (int a = 0; a < 6; ++a) m = imax(m, field(h[a]));
-  const int E = m >> 20;
-  if (E > 1043) return false;
-#pragma unroll
-  for (int a = 0; a < 6; ++a) g.v[a] = conv(h[a], E);
-  g.e = E - 1077;
-  const int one = 1 << (26 - (E - 1023));
-  g.v[0].h += one; g.v[3].h += one; g.v[5].h += one;
-  return true;
-}
-
-// gt^ij as a group and as integers R in units of 2^eR; det gt in units of
-// 2^edet; false where det gt <= 0
-SF_HD bool metric_inverse(const Grp<6> &g, Grp<6> &gi, i64 (&R)[6], int &eR, i64 &det, int &edet) {
-  auto cof = [&](int a, int b, int c, int d) {     // g_a g_b - g_c g_d
-    Acc s;
-    mac(s, g.v[a], g.v[b]);
-    mac(s, -g.v[c], g.v[d]);
-    return fin(s);
-  };
-  R[0] = cof(3, 5, 4, 4);
-  R[1] = cof(2, 4, 1, 5);
-  R[2] = cof(1, 4, 2, 3);
-  R[3] = cof(0, 5, 2, 2);
-  R[4] = cof(1, 2, 0, 4);
-  R[5] = cof(0, 3, 1, 1);
-  Grp<6> c;
-  norm(R, 2 * g.e + kUnit, c);
-  Acc s;
-  mac(s, g.v[0], c.v[0]);
-  mac(s, g.v[1], c.v[1]);
-  mac(s, g.v[2], c.v[2]);
-  det = fin(s);
-  edet = g.e + c.e + kUnit;
-  if (det <= 0) return false;
-  const int n = clz64((u64)det);                   // det = m 2^(63 - n + edet), m in [1, 2)
-  const u64 u = (u64)det << n;
-  u64 M = (u >> 11) + ((u >> 10) & 1);
-  M = M >> 53 ? (1ull << 53) - 1 : M;
-  const i64 iv = rcp62((unsigned)(M >> 32), (unsigned)M) >> 7;   // at most 2^55
-  const Bf idet = Bf{(int)(iv >> 28), (int)((unsigned)iv & 0xFFFFFFFu)};
-#pragma unroll
-  for (int a = 0; a < 6; ++a) {
-    Acc q;
-    mac(q, c.v[a], idet);
-    R[a] = fin(q);
-  }
-  eR = c.e - 55 - (63 - n + edet) + kUnit;
-  norm(R, eR, gi);
-  return true;
 }
 
 }  // namespace sf

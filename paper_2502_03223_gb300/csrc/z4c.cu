@@ -10,7 +10,7 @@
 #include "kernels.h"
 #include "z4c.cuh"
 #include "fixed.cuh"
-#include "z4c_fx.cuh"
+#include "z4c_pass.cuh"
 
 namespace sacra {
 
@@ -1078,79 +1078,63 @@ __device__ inline void load_z4c_in(const Lev &L, const double *__restrict__ U, c
   }
 }
 
-template <typename T>
-__device__ __forceinline__ void z4c_point_cell(const Lev &L, const DevParams &p, const double *__restrict__ U,
-                                                    const T *__restrict__ DS, int jmax, int kmax, int j, int k,
-                                                    double *__restrict__ rs_out = nullptr) {
+// The FP32 form of the mixed precision (the FP64 form: z4c_cell_a, z4c_cell_b)
+__device__ __forceinline__ void z4c_point_f32_cell(const Lev &L, const DevParams &p, const double *__restrict__ U,
+                                                   const float *__restrict__ DS, int jmax, int kmax, int j, int k,
+                                                   double *__restrict__ rs_out) {
   if (j > jmax || k > kmax) return;
   const size_t P = L.P;
   const int id = cid(L, j, k);
-  Z4cIn<T> z;
+  Z4cIn<float> z;
   load_z4c_in(L, U, DS, id, z);
-  Geo<T> G;
+  Geo<float> G;
   geo_fill(z, G);
   geo_ricci(z, G);
-  if (rs_out) rs_out[id] = to_f64<T>(G.Rs);
-  T pr[NPRIM];
+  if (rs_out) rs_out[id] = to_f64<float>(G.Rs);
+  float pr[NPRIM];
 #pragma unroll
-  for (int f = 0; f < NPRIM; ++f) pr[f] = ld_as<T>(L.prim[(size_t)f * P + id]);
-  T E, Si[3], Sij[6];
+  for (int f = 0; f < NPRIM; ++f) pr[f] = ld_as<float>(L.prim[(size_t)f * P + id]);
+  float E, Si[3], Sij[6];
   matter(pr, z.W, G.g, G.gi, E, Si, Sij);
-  T fz;
-  if constexpr (sizeof(T) == 4) {
-    const float x = ((float)j - 0.5f) * f32_of(L.dx), zc = ((float)k - 0.5f) * f32_of(L.dz);
-    fz = expf(-(x * x + zc * zc) * p.firz2);
-  } else {
-    const double x = (j - 0.5) * L.dx, zc = (k - 0.5) * L.dz;
-    fz = exp(-(x * x + zc * zc) / (p.r_z4 * p.r_z4));
-  }
-  T src[NMET];
+  const float x = ((float)j - 0.5f) * f32_of(L.dx), zc = ((float)k - 0.5f) * f32_of(L.dz);
+  const float fz = expf(-(x * x + zc * zc) * p.firz2);
+  float src[NMET];
   z4c_source(p, z, G, E, Si, Sij, fz, src);
+  // source + advection / KO, their FP32 sum widened exactly
 #pragma unroll
-  // FP64: source + advection/KO in FP64; FP32: their FP32 sum, widened exactly
-#pragma unroll
-  for (int f = 0; f < NMET; ++f) L.rhs[(size_t)f * P + id] = to_f64<T>(src[f] + DS[(size_t)(DS_AK + f) * P + id]);
+  for (int f = 0; f < NMET; ++f) L.rhs[(size_t)f * P + id] = to_f64<float>(src[f] + DS[(size_t)(DS_AK + f) * P + id]);
 }
 
-// cells the block fixed-point form hands back (non-finite values): out of
-// line, so that its registers do not weigh on the other path
-__device__ __noinline__ void z4c_point_fp64(const Lev &L, const DevParams &p, const double *__restrict__ U,
-                                            const double *__restrict__ DS, int jmax, int kmax, int j, int k,
-                                            double *__restrict__ rs_out) {
-  z4c_point_cell<double>(L, p, U, DS, jmax, kmax, j, k, rs_out);
-}
-
-// The FP64 right-hand side of a cell in block fixed point (z4c_fx.cuh), its
-// second pass handing cells back to the FP64 algebra.  Pass A's results wait
-// in the right-hand side's planes.
-__device__ __forceinline__ void z4c_cell_fx_a(const Lev &L, const double *__restrict__ U, const double *__restrict__ DS,
-                                              int jmax, int kmax, int j, int k) {
+// The two FP64 passes of a cell (z4c_pass.cuh).  Pass A's results wait in the
+// right-hand side's planes.
+__device__ __forceinline__ void z4c_cell_a(const Lev &L, const double *__restrict__ U, const double *__restrict__ DS,
+                                           int jmax, int kmax, int j, int k) {
   if (j > jmax || k > kmax) return;
   const size_t P = L.P;
   const int id = cid(L, j, k);
   const double *u = U + id, *ds = DS + id;
   double *r = L.rhs + id;
-  z4c_fx_a([&](int f) { return u[(size_t)f * P]; }, [&](int a, int q) { return ds[(size_t)(DS_D1 + 3 * a + q) * P]; },
-           [&](int f, double v) { r[(size_t)f * P] = v; });
+  z4c_pass_a<double>([&](int f) { return u[(size_t)f * P]; },
+                     [&](int a, int q) { return ds[(size_t)(DS_D1 + 3 * a + q) * P]; },
+                     [&](int f, double v) { r[(size_t)f * P] = v; });
 }
 
-__device__ __forceinline__ void z4c_cell_fx_b(const Lev &L, const DevParams &p, const double *__restrict__ U,
-                                              const double *__restrict__ DS, int jmax, int kmax, int j, int k,
-                                              double *__restrict__ rs_out) {
+__device__ __forceinline__ void z4c_cell_b(const Lev &L, const DevParams &p, const double *__restrict__ U,
+                                           const double *__restrict__ DS, int jmax, int kmax, int j, int k,
+                                           double *__restrict__ rs_out) {
   if (j > jmax || k > kmax) return;
   const size_t P = L.P;
   const int id = cid(L, j, k);
   const double x = (j - 0.5) * L.dx, zc = (k - 0.5) * L.dz;
   const double fz = exp(-t_div(x * x + zc * zc, p.r_z4 * p.r_z4));
-  const Z4cPar zp{p.kappa, p.eta_B, p.bssn};
+  const Z4cPar<double> zp{p.kappa, p.eta_B, p.bssn};
   const double *u = U + id, *ds = DS + id, *pr = L.prim + id;
   double *r = L.rhs + id;
-  const bool ok = z4c_fx_b(
+  z4c_pass_b<double>(
       zp, [&](int f) { return u[(size_t)f * P]; }, [&](int a, int q) { return ds[(size_t)(DS_D1 + 3 * a + q) * P]; },
       [&](int a, int q) { return ds[(size_t)(DS_D2 + 6 * a + q) * P]; }, [&](int f) { return ds[(size_t)(DS_AK + f) * P]; },
       [&](int f) { return pr[(size_t)f * P]; }, [&](int f) { return r[(size_t)f * P]; }, fz,
-      [&](int f, double v) { r[(size_t)f * P] = v; }, rs_out ? rs_out + id : nullptr);
-  if (!ok) z4c_point_fp64(L, p, U, DS, jmax, kmax, j, k, rs_out);
+      [&](int f, double v) { r[(size_t)f * P] = v; }, [&](double v) { if (rs_out) rs_out[id] = v; });
 }
 
 // ---------------------------------------------------------------- host launchers
@@ -1213,19 +1197,19 @@ __global__ void __launch_bounds__(FDX * FDZ, 4) kb_z4c_derivs(Batch b, DevParams
   });
 }
 
-// Pass A needs its 255 registers (3 blocks per SM: 40 % slower, spills), pass
-// B hides its loads better with four blocks per SM (7.3 ms per step of the
-// migration star for both passes, 7.4 with three, 8.0 with two).
+// Both passes are bound by the FP64 pipe.  Pass A takes 240 registers (3 blocks
+// per SM: spills, 10.0 ms for both passes per step of the migration star
+// 5 x 512^2, against 9.8), pass B is the same with 3 or 4 blocks per SM.
 __global__ void __launch_bounds__(128, 2) kb_z4c_point_a(Batch b) {
   for_tiles<false>(b, [&](const BL &q, const Tile &tl) {
-    z4c_cell_fx_a(q.L, q.U, reinterpret_cast<const double *>(q.DS), q.jmax, q.kmax, tl.j0 + threadIdx.x, tl.k0 + threadIdx.y);
+    z4c_cell_a(q.L, q.U, reinterpret_cast<const double *>(q.DS), q.jmax, q.kmax, tl.j0 + threadIdx.x, tl.k0 + threadIdx.y);
   });
 }
 
 __global__ void __launch_bounds__(128, 4) kb_z4c_point_b(Batch b, int store_rs) {
   for_tiles<false>(b, [&](const BL &q, const Tile &tl) {
     double *rs = store_rs ? reinterpret_cast<double *>(q.DS) + (size_t)DS_RS * q.L.P : nullptr;
-    z4c_cell_fx_b(q.L, q.P, q.U, reinterpret_cast<const double *>(q.DS), q.jmax, q.kmax, tl.j0 + threadIdx.x,
+    z4c_cell_b(q.L, q.P, q.U, reinterpret_cast<const double *>(q.DS), q.jmax, q.kmax, tl.j0 + threadIdx.x,
                   tl.k0 + threadIdx.y, rs);
   });
 }
@@ -1233,7 +1217,7 @@ __global__ void __launch_bounds__(128, 4) kb_z4c_point_b(Batch b, int store_rs) 
 __global__ void __launch_bounds__(128, 4) kb_z4c_point_f32(Batch b, int store_rs) {
   for_tiles<false>(b, [&](const BL &q, const Tile &tl) {
     double *rs = store_rs ? reinterpret_cast<double *>(q.DS) + (size_t)DS_RS * q.L.P : nullptr;
-    z4c_point_cell<float>(q.L, q.P, q.U, reinterpret_cast<const float *>(q.DS), q.jmax, q.kmax, tl.j0 + threadIdx.x,
+    z4c_point_f32_cell(q.L, q.P, q.U, reinterpret_cast<const float *>(q.DS), q.jmax, q.kmax, tl.j0 + threadIdx.x,
                           tl.k0 + threadIdx.y, rs);
   });
 }
