@@ -219,7 +219,6 @@ struct Engine {
   char *arena = nullptr;
   bool own_arena = false;
   double *tab = nullptr, *tabw = nullptr, *dout = nullptr;
-  CartoonFx cfx{nullptr, nullptr, 0};
   unsigned long long *nfb = nullptr;
   int *tctr = nullptr;            // the tile counters of the batched launches, one per kind (zeroed per stage)
   int sms = 1;
@@ -596,7 +595,7 @@ void launch_kind(Engine &e, int kind, const Batch &b, int s, double dt, cudaStre
     case B_FLUX_X: launch_b_flux_x(b, e.dp, st); break;
     case B_FLUX_Z: launch_b_flux_z(b, e.dp, st); break;
     case B_HYDRO: launch_b_hydro_div(b, e.dp, st); break;
-    case B_CARTOON: launch_b_cartoon(b, e.dp, e.tab, kTabStride, e.tabw, e.cfx, st); break;
+    case B_CARTOON: launch_b_cartoon(b, e.dp, e.tab, kTabStride, e.tabw, st); break;
     case B_DERIVS: launch_b_z4c_derivs(b, e.dp, st); break;
     case B_POINT: launch_b_z4c_point(b, e.dp, st, s == 0 && e.stage0_diag ? 1 : 0); break;
     case B_RK: launch_b_rk_update(b, e.dp, s, dt, st); break;
@@ -1116,43 +1115,6 @@ void upload_tables(Engine &e, int max_nx) {
       W[64] += 2.0 * w2[m] * sn * sn;
     }
   }
-  // the weights on a fixed-point grid per column and array (kernels.h): |w| < 2^54 units,
-  // each rounded once; the centre's weight in Sd, C2, F, G, H takes what makes the array add
-  // up to 0, K2, -Kb, Kb and -2 Kb
-  std::vector<int2> wi((size_t)nj * kCartoonI, make_int2(0, 0));
-  std::vector<int> we((size_t)nj * kCartoonE, 0);
-  for (int j = 1; j < nj; ++j) {
-    const double *Wd = &tw[(size_t)j * kCartoonW];
-    const double K2 = Wd[63], Kb = Wd[64];
-    const bool folded[7] = {true, false, false, true, true, true, true};
-    const double total[7] = {0.0, 0.0, 0.0, K2, -Kb, Kb, -2.0 * Kb};
-    double mx[7];
-    for (int s = 0; s < 7; ++s) {
-      // a bound on every weight: the sum of the others' magnitudes and the total bound the centre's
-      double m = fabs(total[s]);
-      for (int n = 0; n < 9; ++n) m += fabs(Wd[9 * s + n]);
-      mx[s] = m;
-    }
-    mx[4] = mx[5] = std::max(mx[4], mx[5]);
-    for (int s = 0; s < 7; ++s) {
-      int ex;
-      frexp(mx[s], &ex);                            // mx < 2^ex
-      const int e = ex - 54;
-      long long sum = 0, q[9];
-      for (int n = 0; n < 9; ++n) {
-        q[n] = llrint(ldexp(Wd[9 * s + n], -e));
-        if (n != 4) sum += q[n];
-      }
-      if (folded[s]) q[4] = llrint(ldexp(total[s], -e)) - sum;
-      for (int n = 0; n < 9; ++n) {
-        const long long h = q[n] >> 28;
-        wi[(size_t)(9 * s + n) * nj + j] = make_int2((int)h, (int)(q[n] - h * (1ll << 28)));
-      }
-      we[(size_t)s * nj + j] = e;
-    }
-  }
-  cudaMemcpyAsync(const_cast<int2 *>(e.cfx.w), wi.data(), wi.size() * sizeof(int2), cudaMemcpyHostToDevice, e.stream);
-  cudaMemcpyAsync(const_cast<int *>(e.cfx.e), we.data(), we.size() * sizeof(int), cudaMemcpyHostToDevice, e.stream);
   cudaMemcpyAsync(e.tab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice, e.stream);
   cudaMemcpyAsync(e.tabw, tw.data(), tw.size() * sizeof(double), cudaMemcpyHostToDevice, e.stream);
   GridWeights w;
@@ -1177,11 +1139,6 @@ size_t litem_count(const std::vector<sacra_params> &ps) {
   return n;
 }
 
-// the cartoon weights in block fixed point (limbs, then exponents)
-size_t cartoon_fx_bytes_of(int max_nx) {
-  return round_up((size_t)(max_nx + 8) * (kCartoonI * sizeof(int2) + kCartoonE * sizeof(int)), 256);
-}
-
 size_t engine_bytes(const std::vector<sacra_params> &ps) {
   size_t n = 0;
   int max_nx = 0;
@@ -1189,8 +1146,7 @@ size_t engine_bytes(const std::vector<sacra_params> &ps) {
     n += star_bytes(&p);
     max_nx = std::max(max_nx, p.nx);
   }
-  return n + round_up((size_t)(max_nx + 8) * (3 * kTabStride + kCartoonW) * 8, 256) + cartoon_fx_bytes_of(max_nx) +
-         256 /* dout */ + 256 /* nfb */ +
+  return n + round_up((size_t)(max_nx + 8) * (3 * kTabStride + kCartoonW) * 8, 256) + 256 /* dout */ + 256 /* nfb */ +
          256 /* tile counter */ +
          plan_bytes(ps) + round_up(litem_count(ps) * sizeof(LItem), 256);
 }
@@ -1267,10 +1223,6 @@ sacra_status engine_init(Engine &e, const std::vector<sacra_params> &ps, void *s
   e.tab = (double *)p;
   e.tabw = e.tab + (size_t)(max_nx + 8) * 3 * kTabStride;
   p += round_up((size_t)(max_nx + 8) * (3 * kTabStride + kCartoonW) * 8, 256);
-  e.cfx.n = max_nx + 8;
-  e.cfx.w = (const int2 *)p;
-  e.cfx.e = (const int *)(p + (size_t)e.cfx.n * kCartoonI * sizeof(int2));
-  p += cartoon_fx_bytes_of(max_nx);
   e.dout = (double *)p;
   p += 256;
   e.nfb = (unsigned long long *)p;
@@ -1475,7 +1427,7 @@ void enqueue_diag(Engine &e, Star &st, bool own_derivs) {
     const long long cells = (long long)lv.nx * lv.nz;
     double *ds = reinterpret_cast<double *>(st.ds[l]);
     if (own_derivs && st.prm.evolve_spacetime) {
-      run(e, K_CARTOON, (long long)(lv.nx + 7) * (lv.nz + 10), [&] { launch_cartoon(lv, st.dp, lv.un, e.tab, kTabStride, e.tabw, e.cfx, e.stream); });
+      run(e, K_CARTOON, (long long)(lv.nx + 7) * (lv.nz + 10), [&] { launch_cartoon(lv, st.dp, lv.un, e.tab, kTabStride, e.tabw, e.stream); });
       run(e, K_Z4C_DERIVS, cells, [&] { launch_z4c_derivs(lv, st.dp, lv.un, ds, lv.nx, lv.nz, e.stream); });
     }
     const int sl = slot;

@@ -109,19 +109,8 @@ void launch_b_hydro_div(const Batch &b, const DevParams &p, cudaStream_t s);
 // differences over the planes m = -3..3 folded together), dimensionless:
 //   [0, 9) Sd, [9, 18) D1, [18, 27) E1, [27, 36) C2, [36, 45) F, [45, 54) G, [54, 63) H, 63 K2, 64 Kb
 constexpr int kCartoonW = 68;
-// The same weights in block fixed point (softfp.cuh) for the kernel's integer
-// sums, slot-major over the columns: slots [0, 63) the limbs of Sd, D1, E1, C2,
-// F, G, H with the terms on the centre value folded into its weight (Sd, C2, F,
-// G, H act on u_n, not u_n - u_0: the weights of a derivative of a constant add
-// up to zero exactly, in integers), then kCartoonE exponents (F and G share theirs)
-constexpr int kCartoonI = 63, kCartoonE = 7;
-struct CartoonFx {
-  const int2 *w;       // [kCartoonI][n]
-  const int *e;        // [kCartoonE][n]
-  int n;               // columns of the table
-};
 void launch_b_cartoon(const Batch &b, const DevParams &p, const double *tab, int tab_stride, const double *tabw,
-                      const CartoonFx &fx, cudaStream_t s);
+                      cudaStream_t s);
 void launch_b_z4c_derivs(const Batch &b, const DevParams &p, cudaStream_t s);
 // store_rs: the pass also writes the Ricci scalar it forms (FP64, or the FP32
 // value widened) into the FP64 scratch plane z4c_ricci_plane()
@@ -143,7 +132,7 @@ void launch_c2p_region(const Lev &L, const DevParams &p, double *U, int j0, int 
                        int skip_corner = 0);
 
 void launch_cartoon(const Lev &L, const DevParams &p, const double *U, const double *tab, int tab_stride,
-                    const double *tabw, const CartoonFx &fx, cudaStream_t s);
+                    const double *tabw, cudaStream_t s);
 void launch_z4c_derivs(const Lev &L, const DevParams &p, const double *U, double *DS, int jmax, int kmax, cudaStream_t s);
 int z4c_scratch_planes();
 int z4c_ricci_plane();

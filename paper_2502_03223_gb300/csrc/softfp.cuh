@@ -61,13 +61,6 @@ SF_HD unsigned hiw(i64 b) { return (unsigned)((u64)b >> 32); }
 SF_HD unsigned low(i64 b) { return (unsigned)b; }
 SF_HD unsigned umulhi32(unsigned a, unsigned b) { return (unsigned)(((u64)a * b) >> 32); }
 SF_HD i64 wide(int a, int b) { return (i64)a * b; }
-SF_HD int clz64(u64 x) {
-#ifdef __CUDA_ARCH__
-  return __clzll((i64)x);
-#else
-  return x ? __builtin_clzll(x) : 64;
-#endif
-}
 // FP32 seeds (the hardware approximations; the host form is for tests)
 SF_HD float seed_rcp(float f) {
 #ifdef __CUDA_ARCH__
@@ -234,40 +227,6 @@ SF_HD double srsqrt(double a) {
   i64 M; float f; int k;
   root_parts(b, M, f, k);
   return pack61((u64)(rsqrt62(M, f) >> 1), 1023 - k, 0u);
-}
-
-// ---------------------------------------------------------------- parts of integer sums
-
-SF_HD u64 shr_clamp(u64 u, int k) {              // u / 2^k, 0 for k >= 64
-#ifdef __CUDA_ARCH__
-  u64 r; asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(u), "r"(k)); return r;
-#else
-  return k < 64 ? u >> k : 0;
-#endif
-}
-SF_HD int field(double x) { return (int)(hiw(bits(x)) & 0x7FFFFFFFu); }   // exponent and top fraction bits
-
-// R 2^e as a double, rounded to nearest; results below the normal range are
-// zero, above it infinite
-SF_HD double to_double(i64 R, int e) {
-#if defined(__CUDA_ARCH__)
-  // one FP64 conversion, the exponent by an integer addition
-  const i64 b = bits((double)R);
-  const int er = (int)(hiw(b) >> 20) & 0x7FF;
-  if (er == 0) return 0.0;
-  if ((unsigned)(er + e - 1) >= 2045u) return er + e < 1 ? 0.0 : of_bits((b & (i64)(1ull << 63)) | 0x7FF0000000000000ll);
-  return of_bits(b + ((i64)e << 52));
-#else
-  const u64 s = (u64)(R >> 63);
-  const u64 a = ((u64)R ^ s) - s;
-  const int n = clz64(a);
-  const u64 u = a << (n & 63);
-  const int ex = 1086 - n + e;
-  const u64 m = (u >> 11) + ((u >> 10) & 1);        // 53 bits with the leading one (or the next power of two)
-  u64 b = m + ((u64)(unsigned)(ex - 1) << 52);
-  if ((unsigned)(ex - 1) >= 2045u || n == 64) b = (n == 64 || ex < 1) ? 0ull : 0x7FF0000000000000ull;
-  return of_bits((i64)(b | (s << 63)));
-#endif
 }
 
 }  // namespace sf

@@ -34,9 +34,6 @@ __host__ __device__ constexpr float par_x_slot(int a) {
              ? -1.0f : 1.0f;
 }
 
-// the first of a tile's stencil columns, (smallest jj of the tile) - 4
-__device__ __forceinline__ int cartoon32_base(int j0) { return (j0 >= 1 ? j0 : 1) - 4; }
-
 // d_y and d_yy at (x_j, z_k) by the cartoon method (Sec. II.B.2): the planes
 // y = +-m dy (m = 1..3, dy = dx) hold the 9-point Lagrange interpolant in x at
 // varpi_m = sqrt(x_j^2 + (m dy)^2), rotated by +-phi_m, and d_y, d_yy are the
@@ -139,195 +136,8 @@ __device__ __forceinline__ void cartoon_f64_cell(const Lev &L, const double *__r
   }
 }
 
-// The FP64 planes as integer sums.  In FP64 the kernel kept its pipe 88 % busy
-// with 430 instructions per warp at 16 cycles each.  Here a cell puts the nine
-// values of each field's stencil on one fixed-point grid (58 bits below their
-// largest exponent, so a value within a factor 32 of it keeps its 53 bits);
-// every output is a sum of nine exact products of two-limb integers (four
-// mad.wide each), and the sum (up to 116 bits) is rounded once, scaled once.
-// The grid is the stencil's own, so a plane's values depend on nothing but the
-// values they are made of.  (One grid per row segment of a tile is faster, 1.6
-// instead of 1.9 ms per step, but ties a cell to its tile and to far values;
-// one per four columns cost more than it saved.)  A stencil with a non-finite
-// value takes the FP64 form.  3.94 -> 1.91 ms per step of the migration star
-// (5 x 512^2).
-enum : int { cW = 0, cAL, cHXX, cHXY, cHXZ, cHYY, cHYZ, cHZZ, cAXX, cAXY, cAXZ, cAYY, cAYZ, cBX, cBY, cBZ, cGX, cGY, cQX, cQY };
-// shared memory: the tile's values [field][row][column], columns from cartoon32_base(j0)
-__host__ __device__ constexpr int cartoon_fx_bytes(int bx, int by) { return 20 * by * (bx + 8) * (int)sizeof(double); }
-
-// v = u 2^(E - 1080)^-1, |v| < 2^58, as limbs h 2^28 + l
-__device__ __forceinline__ int2 cartoon_fix(double x, int E) {
-  const sf::i64 b = sf::bits(x);
-  const unsigned hi = sf::hiw(b), lo = sf::low(b);
-  const sf::u64 u = ((sf::u64)(((hi << 11) | (lo >> 21)) | 0x80000000u) << 32) | (lo << 11);
-  const sf::u64 v = sf::shr_clamp(u, 6 + E - (int)((hi >> 20) & 0x7FFu));
-  const int s = ((int)hi >> 31) | 1;
-  return make_int2((int)(v >> 28) * s, (int)((unsigned)v & 0xFFFFFFFu) * s);
-}
-
-__device__ __forceinline__ void cartoon_fx_stage(const Lev &L, const double *__restrict__ U, int j0, int k0, double *sm) {
-  const int bx = (int)blockDim.x, by = (int)blockDim.y, nc = bx + 8, per = by * nc;
-  const int nth = bx * by, tid = (int)(threadIdx.y * blockDim.x + threadIdx.x);
-  const int base = cartoon32_base(j0);
-  for (int e = tid; e < per; e += nth) {              // one stencil point per thread and pass, its 20 fields together
-    const int j = base + e % nc, k = k0 + e / nc;
-    if (j > L.nx + GH || k > L.nz + 7) continue;      // past every stencil of the region's cells
-    const int id = cid(L, j, k);
-    double u[20];
-#pragma unroll
-    for (int a = 0; a < 20; ++a) u[a] = U[(size_t)kCartoonFields[a] * L.P + id];
-#pragma unroll
-    for (int a = 0; a < 20; ++a) sm[a * per + e] = u[a];
-  }
-  __syncthreads();
-}
-
-// exact sum of products of limbs: (H 2^56 + C 2^28 + Lo) 2^(ex + ey)
-struct Acc3 {
-  sf::i64 H = 0, C = 0, Lo = 0;
-};
-__device__ __forceinline__ void mac4(Acc3 &a, int2 x, int2 y) {
-  a.H += sf::wide(x.x, y.x);
-  a.C += sf::wide(x.x, y.y);
-  a.C += sf::wide(x.y, y.x);
-  a.Lo += sf::wide(x.y, y.y);
-}
-// the sum rounded to a double: its leading 63 bits, converted once
-__device__ __forceinline__ double acc3_double(const Acc3 &s, int e) {
-  const sf::i64 a = s.C + (s.Lo >> 28);
-  const sf::i64 b = s.H + (a >> 28);
-  const sf::u64 r = ((sf::u64)(a & 0xFFFFFFF) << 28) | (sf::u64)(s.Lo & 0xFFFFFFF);   // T = b 2^56 + r, 0 <= r < 2^56
-  const int n = min(__clzll((long long)((b ^ (b >> 63)) | 1)) - 2, 56);
-  const sf::i64 v = (sf::i64)((sf::u64)b << n) + (sf::i64)(r >> (56 - n));
-  return sf::to_double(v, e + 56 - n);
-}
-
-__device__ __noinline__ void cartoon_f64_row(const Lev &L, const double *__restrict__ U, const double *__restrict__ tabw,
-                                             int j, int k) {
-  cartoon_f64_cell(L, U, tabw, j, k);
-}
-
-__device__ __forceinline__ void cartoon_fx_cell(const Lev &L, const double *__restrict__ U, const double *__restrict__ tabw,
-                                                const CartoonFx &fx, int j0, int j, int k, const double *sm) {
-  if (j > L.nx + 4 || k > L.nz + 7) return;
-  const int nc = (int)blockDim.x + 8, per = (int)blockDim.y * nc;
-  const bool flip = j <= 0;
-  const int jj = flip ? 1 - j : j;
-  const size_t P = L.P;
-  const int o = cid(L, j, k);
-  const double *v = sm + (int)threadIdx.y * nc + (jj - 4 - cartoon32_base(j0));   // field a: + a per
-  const double i1 = L.i60x, i2 = L.i180x;
-  int top = 0;                                      // the largest exponent field seen
-  int2 x[9], D1[9], w[9];
-  int ex = 0, e1 = 0, we = 0;
-  auto weights = [&](int s, int2 (&q)[9], int &e) { // weight array s (Sd, D1, E1, C2, F, G, H)
-#pragma unroll
-    for (int n = 0; n < 9; ++n) q[n] = fx.w[(size_t)(9 * s + n) * fx.n + jj];
-    e = fx.e[(size_t)s * fx.n + jj];
-  };
-  auto take = [&](int a) {                          // field a's stencil on its grid
-    double u[9];
-    int m = 64 << 20;
-#pragma unroll
-    for (int n = 0; n < 9; ++n) {
-      u[n] = v[a * per + n];
-      m = max(m, sf::field(u[n]));
-    }
-    const int E = m >> 20;
-    top = max(top, E);
-    ex = E - 1080;
-#pragma unroll
-    for (int n = 0; n < 9; ++n) x[n] = cartoon_fix(u[n], E);
-  };
-  auto dot = [&](Acc3 &s, const int2 (&p)[9], const int2 (&q)[9]) {
-#pragma unroll
-    for (int n = 0; n < 9; ++n) mac4(s, p[n], q[n]);
-  };
-  auto sum = [&](const int2 (&q)[9], int e) {
-    Acc3 s;
-    dot(s, x, q);
-    return acc3_double(s, e + ex);
-  };
-  auto st1 = [&](int f, double y) { L.dy[(size_t)f * P + o] = (flip ? -par_x(f) * y : y) * i1; };
-  auto st2 = [&](int f, double y) { L.dyy[(size_t)f * P + o] = (flip ? par_x(f) * y : y) * i2; };
-  weights(0, w, we);                                // d_yy of scalars
-  take(cW);  st2(fW, sum(w, we));
-  take(cAL); st2(fAL, sum(w, we));
-  take(cHZZ); st2(fHZZ, sum(w, we));
-  take(cBZ); st2(fBZ, sum(w, we));
-  // d_y of vectors, T_xz and T_yz from the other component; d_yy of beta^x, beta^y, h_xz, h_yz
-  weights(1, D1, e1);
-  weights(3, w, we);
-  take(cBX);  st1(fBY, -sum(D1, e1)); st2(fBX, sum(w, we));
-  take(cBY);  st1(fBX, sum(D1, e1)); st2(fBY, sum(w, we));
-  take(cHXZ); st1(fHYZ, -sum(D1, e1)); st2(fHXZ, sum(w, we));
-  take(cHYZ); st1(fHXZ, sum(D1, e1)); st2(fHYZ, sum(w, we));
-  take(cGX);  st1(fGY, -sum(D1, e1));
-  take(cGY);  st1(fGX, sum(D1, e1));
-  take(cQX);  st1(fBBY, -sum(D1, e1));
-  take(cQY);  st1(fBBX, sum(D1, e1));
-  take(cAXZ); st1(fAYZ, -sum(D1, e1));
-  take(cAYZ); st1(fAXZ, sum(D1, e1));
-  // d_y of T_xx, T_yy, T_xy; d_yy of h_xy, h_xx, h_yy
-  weights(2, D1, e1);
-  weights(6, w, we);
-  {
-    take(cAXY);
-    const double y = sum(D1, e1);
-    st1(fAXX, y);
-    st1(fAYY, -y);
-  }
-  {
-    take(cHXY);
-    const double y = sum(D1, e1);
-    st1(fHXX, y);
-    st1(fHYY, -y);
-    st2(fHXY, sum(w, we));
-  }
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {                     // (xx, yy) on one grid
-    const int a = q == 0 ? cAXX : cHXX;
-    double u[18];
-    int m = 64 << 20;
-#pragma unroll
-    for (int n = 0; n < 9; ++n) {
-      u[n] = v[a * per + n];
-      u[9 + n] = v[(a + 3) * per + n];
-      m = max(m, max(sf::field(u[n]), sf::field(u[9 + n])));
-    }
-    const int E = m >> 20;
-    top = max(top, E);
-    ex = E - 1080;
-    int2 y[9];
-    Acc3 s;
-#pragma unroll
-    for (int n = 0; n < 9; ++n) {
-      x[n] = cartoon_fix(u[n], E);
-      y[n] = cartoon_fix(u[9 + n], E);
-      mac4(s, make_int2(x[n].x - y[n].x, x[n].y - y[n].y), D1[n]);
-    }
-    st1(q == 0 ? fAXY : fHXY, -0.5 * acc3_double(s, e1 + ex));
-    if (q == 1) {
-      Acc3 sx, sy;
-      weights(4, w, we);
-      dot(sx, x, w);
-      dot(sy, y, w);
-      weights(5, w, we);                            // the exponent of F
-      dot(sx, y, w);
-      dot(sy, x, w);
-      st2(fHXX, acc3_double(sx, we + ex));
-      st2(fHYY, acc3_double(sy, we + ex));
-    }
-  }
-  if (top >= 2047) cartoon_f64_row(L, U, tabw, j, k);   // a non-finite value: overwrite with the FP64 form
-}
-
-__global__ void __launch_bounds__(128) k_cartoon_f64(Lev L, const double *__restrict__ U, const double *__restrict__ tabw,
-                                                     CartoonFx fx) {
-  extern __shared__ double cfx_sm[];
-  const int j0 = (int)(blockIdx.x * blockDim.x) - 2, k0 = (int)(blockIdx.y * blockDim.y) - 2;
-  cartoon_fx_stage(L, U, j0, k0, cfx_sm);
-  cartoon_fx_cell(L, U, tabw, fx, j0, j0 + (int)threadIdx.x, k0 + (int)threadIdx.y, cfx_sm);
+__global__ void __launch_bounds__(128) k_cartoon_f64(Lev L, const double *__restrict__ U, const double *__restrict__ tabw) {
+  cartoon_f64_cell(L, U, tabw, blockIdx.x * blockDim.x + threadIdx.x - 2, blockIdx.y * blockDim.y + threadIdx.y - 2);
 }
 
 // Mixed precision: the same planes in FP32, formed as differences from the
@@ -372,6 +182,7 @@ struct Cartoon32Staged {
 
 // the tile's stencil columns, base = (smallest jj of the tile) - 4 .. base + bx + 7
 __host__ __device__ constexpr int cartoon32_tile_floats(int bx, int by) { return 2 * 20 * by * (bx + 8); }
+__device__ __forceinline__ int cartoon32_base(int j0) { return (j0 >= 1 ? j0 : 1) - 4; }
 
 __device__ __forceinline__ void cartoon32_tile(const Lev &L, const double *__restrict__ U, int j0, int k0, float *sm) {
   const int bx = (int)blockDim.x, by = (int)blockDim.y, nc = bx + 8, per = by * nc;
@@ -1140,10 +951,10 @@ __device__ __forceinline__ void z4c_cell_b(const Lev &L, const DevParams &p, con
 // ---------------------------------------------------------------- host launchers
 
 void launch_cartoon(const Lev &L, const DevParams &p, const double *U, const double *tab, int tab_stride,
-                    const double *tabw, const CartoonFx &fx, cudaStream_t s) {
+                    const double *tabw, cudaStream_t s) {
   dim3 b(32, 4), g((L.nx + 7 + 31) / 32, (L.nz + 10 + 3) / 4);
   if (p.mixed & SACRA_MIXED_Z4C) k_cartoon_f32<<<g, b, 0, s>>>(L, U, tab, tab_stride);
-  else k_cartoon_f64<<<g, b, cartoon_fx_bytes(b.x, b.y), s>>>(L, U, tabw, fx);
+  else k_cartoon_f64<<<g, b, 0, s>>>(L, U, tabw);
 }
 
 void launch_z4c_derivs(const Lev &L, const DevParams &p, const double *U, double *DS, int jmax, int kmax, cudaStream_t s) {
@@ -1158,11 +969,9 @@ void launch_z4c_derivs(const Lev &L, const DevParams &p, const double *U, double
 
 // ---------------------------------------------------------------- batched persistent kernels
 
-__global__ void __launch_bounds__(128, 5) kb_cartoon_f64(Batch b, const double *__restrict__ tabw, CartoonFx fx) {
-  extern __shared__ double cfx_sm[];
+__global__ void __launch_bounds__(128) kb_cartoon_f64(Batch b, const double *__restrict__ tabw) {
   for_tiles(b, [&](const BL &q, const Tile &tl) {
-    cartoon_fx_stage(q.L, q.U, tl.j0, tl.k0, cfx_sm);
-    cartoon_fx_cell(q.L, q.U, tabw, fx, tl.j0, tl.j0 + (int)threadIdx.x, tl.k0 + (int)threadIdx.y, cfx_sm);
+    cartoon_f64_cell(q.L, q.U, tabw, tl.j0 + threadIdx.x, tl.k0 + threadIdx.y);
   });
 }
 
@@ -1223,11 +1032,11 @@ __global__ void __launch_bounds__(128, 4) kb_z4c_point_f32(Batch b, int store_rs
 }
 
 void launch_b_cartoon(const Batch &b, const DevParams &p, const double *tab, int tab_stride, const double *tabw,
-                      const CartoonFx &fx, cudaStream_t s) {
+                      cudaStream_t s) {
   if (b.ntiles <= 0) return;
   if (p.mixed & SACRA_MIXED_Z4C)
     kb_cartoon_f32<<<b.grid, b.block, cartoon32_tile_floats(b.block.x, b.block.y) * sizeof(float), s>>>(b, tab, tab_stride);
-  else kb_cartoon_f64<<<b.grid, b.block, cartoon_fx_bytes(b.block.x, b.block.y), s>>>(b, tabw, fx);
+  else kb_cartoon_f64<<<b.grid, b.block, 0, s>>>(b, tabw);
 }
 
 void launch_b_z4c_derivs(const Batch &b, const DevParams &p, cudaStream_t s) {
