@@ -212,8 +212,8 @@ __device__ __forceinline__ double to_f64(T v) {
 
 // ------------------------------------------------------------------ quotients and roots in arithmetic T
 //
-// FP64: on the integer units (softfp.cuh), 15 to 20 SM cycles per warp instead
-// of 90 to 146 on the FP64 pipe; FP32: the hardware forms.
+// FP64: on the integer units (softfp.cuh), 36 to 57 SM cycles per warp instead
+// of 97 to 151 on the FP64 pipe, which stays free; FP32: the hardware forms.
 __device__ __forceinline__ double t_div(double a, double b) { return sf::sdiv(a, b); }
 __device__ __forceinline__ double t_rcp(double a) { return sf::srcp(a); }
 __device__ __forceinline__ double t_sqrt(double a) { return sf::ssqrt(a); }
@@ -222,6 +222,17 @@ __device__ __forceinline__ float t_div(float a, float b) { return a / b; }
 __device__ __forceinline__ float t_rcp(float a) { return 1.0f / a; }
 __device__ __forceinline__ float t_sqrt(float a) { return sqrtf(a); }
 __device__ __forceinline__ float t_rsqrt(float a) { return rsqrtf(a); }
+
+// d^(-1/3) by one third-order (Householder) step from an FP32 seed:
+// e = 1 - d y0^3, y0 (1 + e/3 + 2/9 e^2); the next term is 14/81 e^3 < 2^-60.
+// Six FP64 operations (rcbrt takes the time of sixteen).
+__device__ __forceinline__ double t_rcbrt(double d) {
+  const int hi = __double2hiint(d);
+  if (hi < 0x3E000000 || hi >= 0x42000000) return rcbrt(d);   // a determinant far from 1, or not a positive number
+  const double y0 = f64_of(exp2f(log2f(f32_of(d)) * (-1.0f / 3.0f)));
+  const double e = fma(-d, y0 * y0 * y0, 1.0);
+  return fma(y0 * e, fma(e, 2.0 / 9.0, 1.0 / 3.0), y0);
+}
 
 // ------------------------------------------------------------------ small tensor helpers
 
@@ -354,7 +365,7 @@ __device__ inline void prim_to_cons(const DevParams &p, const double pr[NPRIM], 
   }
   const double rho = pr[pRHO], P = pr[pP];
   const double rhw = rho * (1.0 + pr[pEPS] + t_div(P, rho)) * w;
-  const double psi6 = sf::sdiv_rn(1.0, W * W * W);   // rounded as the division: D = q W^3 meets rho_atm here
+  const double psi6 = t_rcp(W * W * W);
   q[0] = psi6 * rho * w;
   q[1] = psi6 * rhw * u[0];
   q[2] = psi6 * rhw * u[1] * (p.geometry == SACRA_CYLINDRICAL ? x : 1.0);
@@ -505,8 +516,8 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
     int its, ok;
     const double z = illinois<true>(p, 0.0, r, C2pD{D, t_rcp(D)}, 0.0, r, &its, &ok);
     if (!ok) st |= ST_NOCONV;
-    const double iw = t_rsqrt(1.0 + z * z);
-    const double rho = D * iw;
+    const double w = t_sqrt(1.0 + z * z);
+    const double rho = t_div(D, w);
     const double eps = eos_ec(p, rho), P = eos_pc(p, rho);
     const double iDh = t_rcp(D * (1.0 + eps + t_div(P, rho)));
     pr[pRHO] = rho;
@@ -528,7 +539,7 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
       atomicAdd(p.c2p_stats + 0, 2ull);
       atomicAdd(p.c2p_stats + 3, 1ull);
     }
-    double eps = sf::sdiv_rn(E, D) - 1.0, P;
+    double eps = t_div(E, D) - 1.0, P;
     const double ec = eos_ec(p, D);
     if (less_any(eps, ec)) {
       eps = ec;
@@ -548,7 +559,7 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
   }
   const double iD = t_rcp(D);
   const C2pD Dd{D, iD};
-  const double qq = sf::sdiv_rn(E, D) - 1.0;   // E / D - 1 is near the cold curve's eps: rounded as the division
+  const double qq = t_div(E, D) - 1.0;
   double k = t_div(r, 1.0 + qq);
   const double kmax = p.c2p_kmax;
   if (k > kmax) {

@@ -107,7 +107,7 @@ __device__ __forceinline__ void outer_body(const Lev &L, const double *__restric
   const double x = (j - 0.5) * L.dx, z = (k - 0.5) * L.dz;
   const double r = t_sqrt(x * x + z * z);
   const double fac = 1.0 - t_div(tau, r);
-  const double xi = x * fac * L.idx + 0.5, ze = z * fac * L.idz + 0.5;
+  const double xi = t_div(x * fac, L.dx) + 0.5, ze = t_div(z * fac, L.dz) + 0.5;
   const int i0 = min((int)floor(xi + 0.5), L.nx + GH - 1), k0 = min((int)floor(ze + 0.5), L.nz + GH - 1);
   const double tx = xi - i0, tz = ze - k0;
   const double wx[3] = {0.5 * tx * (tx - 1.0), (1.0 - tx) * (1.0 + tx), 0.5 * tx * (tx + 1.0)};
@@ -273,17 +273,6 @@ __global__ void k_prolong_hydro(Lev L, Lev Pa, DevParams p, double *__restrict__
   prolong_hydro_body(L, Pa, p, U, lo, blockIdx.x);
 }
 
-// d^(-1/3) by one third-order (Householder) step from an FP32 seed:
-// e = 1 - d y0^3, y0 (1 + e/3 + 2/9 e^2); the next term is 14/81 e^3 < 2^-60.
-// Six FP64 operations (rcbrt takes the time of sixteen).
-__device__ __forceinline__ double t_rcbrt(double d) {
-  const int hi = __double2hiint(d);
-  if (hi < 0x3E000000 || hi >= 0x42000000) return rcbrt(d);   // a determinant far from 1, or not a positive number
-  const double y0 = f64_of(exp2f(log2f(f32_of(d)) * (-1.0f / 3.0f)));
-  const double e = fma(-d, y0 * y0 * y0, 1.0);
-  return fma(y0 * e, fma(e, 2.0 / 9.0, 1.0 / 3.0), y0);
-}
-
 // det gt = 1 and tr At = 0 after every stage (Sec. II.B.1):
 // gt <- d^(-1/3) gt, W <- d^(-1/6) W, At <- d^(-1/3)(At - gt tr/3), Khat += tr
 // gi_out, s_out: the inverse of gt before and the factor 1 / c13 = det c13^2
@@ -295,7 +284,7 @@ __device__ __forceinline__ void enforce_algebraic(double &W, double h[6], double
   double det;
   const Sym3 gi = s3inv(g, &det);
   const double tr = gi.xx * A[0] + gi.yy * A[3] + gi.zz * A[5] + 2.0 * (gi.xy * A[1] + gi.xz * A[2] + gi.yz * A[4]);
-  const double c13 = t_rcbrt(det), c16 = t_sqrt(c13), tr3 = tr * (1.0 / 3.0);
+  const double c13 = t_rcbrt(det), c16 = t_sqrt(c13), tr3 = t_div(tr, 3.0);
   const double gv[6] = {g.xx, g.xy, g.xz, g.yy, g.yz, g.zz};
 #pragma unroll
   for (int a = 0; a < 6; ++a) {
@@ -774,7 +763,7 @@ __global__ void __launch_bounds__(DIAG_T) k_diag(Lev L, DevParams p, const S *__
         for (int jj = 0; jj < 3; ++jj)
 #pragma unroll
           for (int m = jj; m < 3; ++m) Au[sp(jj, m)] = Am[jj][0] * gim[0][m] + Am[jj][1] * gim[1][m] + Am[jj][2] * gim[2][m];
-        const double i3W = 3.0 * t_rcp(z.W);
+        const double i3W = t_div(3.0, z.W);
         double M[3];
 #pragma unroll
         for (int ii = 0; ii < 3; ++ii) {

@@ -78,3 +78,28 @@ extern "C" int sacra_probe_split(const double *host_in, int n, float *host_hi, f
   cudaFree(dbuf);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
+
+// Check of the quotients and roots of softfp.cuh (and t_rcbrt) on the device:
+// out holds sdiv(a, b), srcp(b), ssqrt(a), srsqrt(a), t_rcbrt(a), n values each.
+__global__ void k_quotients(const double *a, const double *b, int n, double *out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  out[i] = sacra::t_div(a[i], b[i]);
+  out[(size_t)n + i] = sacra::t_rcp(b[i]);
+  out[2 * (size_t)n + i] = sacra::t_sqrt(a[i]);
+  out[3 * (size_t)n + i] = sacra::t_rsqrt(a[i]);
+  out[4 * (size_t)n + i] = sacra::t_rcbrt(a[i]);
+}
+
+extern "C" int sacra_probe_quotients(const double *host_a, const double *host_b, int n, double *host_out) {
+  if (n <= 0) return -1;
+  double *d = nullptr;
+  if (cudaMalloc(&d, sizeof(double) * 7 * (size_t)n) != cudaSuccess) return -1;
+  double *a = d, *b = d + n, *out = d + 2 * (size_t)n;
+  cudaMemcpy(a, host_a, sizeof(double) * n, cudaMemcpyHostToDevice);
+  cudaMemcpy(b, host_b, sizeof(double) * n, cudaMemcpyHostToDevice);
+  k_quotients<<<(n + 127) / 128, 128>>>(a, b, n, out);
+  cudaMemcpy(host_out, out, sizeof(double) * 5 * (size_t)n, cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  return cudaGetLastError() == cudaSuccess ? 0 : -2;
+}

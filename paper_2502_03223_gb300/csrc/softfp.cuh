@@ -1,16 +1,20 @@
 // FP64 arithmetic on the integer and FP32 units.
 //
 // On this part a warp's FP64 instruction takes 16 cycles of the SM's FP64
-// pipe, a division or square root 90 to 146 (measured, all lanes busy), while
+// pipe, a division or square root 97 to 151 (measured, all lanes busy), while
 // a 32 x 32 + 64-bit integer multiply-add (mad.wide) takes 0.6 and a 32-bit
 // integer operation about 0.5.  The kernels of this library were bound by the
 // FP64 pipe with the integer and FP32 units idle.  sdiv, srcp, ssqrt and
 // srsqrt form the quotient, reciprocal, square root and its reciprocal of
 // doubles there: an FP32 seed (24 bits) and one third-order (Householder) step
 // on the exact residual, all in integers, give 60 bits; the result is then
-// rounded once.  The error is below 0.52 ulp.  Operands outside the normal
-// range (zeros, infinities, NaN, subnormals) and results near its ends take
-// the FP64 instruction sequence.
+// rounded once.  Quotient, reciprocal and square root are corrected by their
+// exact remainder, so they are the correctly rounded ones, bit for bit those
+// of the FP64 instructions (decisions such as rho < rho_atm compare values
+// formed by them); srsqrt is off by less than 0.52 ulp.  Operands outside the
+// normal range (zeros, infinities, NaN, subnormals) and results near its ends
+// take the FP64 instruction sequence.  36 (srcp) to 57 (ssqrt) SM cycles per
+// warp on the integer pipe.
 #pragma once
 
 #include <math.h>
@@ -61,19 +65,22 @@ SF_HD unsigned hiw(i64 b) { return (unsigned)((u64)b >> 32); }
 SF_HD unsigned low(i64 b) { return (unsigned)b; }
 SF_HD unsigned umulhi32(unsigned a, unsigned b) { return (unsigned)(((u64)a * b) >> 32); }
 SF_HD i64 wide(int a, int b) { return (i64)a * b; }
-// FP32 seeds (the hardware approximations; the host form is for tests)
+// FP32 seeds: the hardware approximations (the host form, for tests, may be nudged)
+#ifndef SF_SEED
+#define SF_SEED(f) (f)
+#endif
 SF_HD float seed_rcp(float f) {
 #ifdef __CUDA_ARCH__
   float r; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f)); return r;
 #else
-  return 1.0f / f;
+  return SF_SEED(1.0f / f);
 #endif
 }
 SF_HD float seed_rsqrt(float f) {
 #ifdef __CUDA_ARCH__
   float r; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f)); return r;
 #else
-  return 1.0f / sqrtf(f);
+  return SF_SEED(1.0f / sqrtf(f));
 #endif
 }
 
@@ -154,6 +161,17 @@ SF_HD double slow_rsqrt(double a) {
 #endif
 }
 
+// The correctly rounded quotient ma 2^k / mb (53-bit significands, k = 52 or
+// 53) from its neighbour q (mq its significand, off by less than one unit):
+// q one unit up or down where the remainder exceeds half a divisor.  The
+// remainder is below 2^54, so its low 64 bits hold it; a tie cannot occur.
+SF_HD double round_quotient(double q, u64 ma, u64 mb, int k) {
+  const i64 bq = bits(q);
+  const u64 mq = ((u64)bq & ((1ull << 52) - 1)) | (1ull << 52);
+  const i64 r2 = (i64)((ma << k) - mq * mb) * 2;
+  return of_bits(bq + (r2 > (i64)mb) - (r2 < -(i64)mb));
+}
+
 // a / b
 SF_HD double sdiv(double a, double b) {
   const i64 ba = bits(a), bb = bits(b);
@@ -164,11 +182,14 @@ SF_HD double sdiv(double a, double b) {
       return of_bits((i64)(((u64)ba ^ (u64)bb) & (1ull << 63)));
     return slow_div(a, b);
   }
-  const i64 A = (i64)((((u64)ba & ((1ull << 52) - 1)) | (1ull << 52)) << 9);       // [2^61, 2^62)
-  const i64 r = rcp62((hiw(bb) & 0xFFFFFu) | 0x100000u, low(bb));                  // (2^61, 2^62]
+  const u64 ma = ((u64)ba & ((1ull << 52) - 1)) | (1ull << 52), mb = ((u64)bb & ((1ull << 52) - 1)) | (1ull << 52);
+  const i64 A = (i64)(ma << 9);                                                    // [2^61, 2^62)
+  const i64 r = rcp62((unsigned)(mb >> 32), low(bb));                              // (2^61, 2^62]
   // A r 2^-62 lies in [2^60, 2^62); r may reach 2^62 only for b a power of two
   const i64 Q = mulhi62(A, r - (r >> 62));
-  return pack61((u64)Q, ex, (hiw(ba) ^ hiw(bb)) & 0x80000000u);
+  const double q = pack61((u64)Q, ex, (hiw(ba) ^ hiw(bb)) & 0x80000000u);
+  const int eq = (int)(hiw(bits(q)) >> 20) & 0x7FF;
+  return round_quotient(q, ma, mb, ex - eq + 52);
 }
 
 // 1 / b
@@ -176,27 +197,11 @@ SF_HD double srcp(double b) {
   const i64 bb = bits(b);
   const int eb = (int)(hiw(bb) >> 20) & 0x7FF;
   if ((unsigned)(eb - 3) >= 2040u) return slow_div(1.0, b);
-  const i64 r = rcp62((hiw(bb) & 0xFFFFFu) | 0x100000u, low(bb));
-  return pack61((u64)(r >> 1), 2046 - eb, hiw(bb) & 0x80000000u);
-}
-
-// a / b rounded to nearest as the FP64 division rounds it: the rounded 53-bit
-// quotient q of sdiv is checked by its exact remainder (a - q b lies within
-// half a b, and the low 64 bits hold it).  For decisions that compare values
-// formed this way with a threshold built from the same numbers.
-SF_HD double sdiv_rn(double a, double b) {
-  const double q = sdiv(a, b);
-  const i64 ba = bits(a), bb = bits(b), bq = bits(q);
-  const int ea = (int)(hiw(ba) >> 20) & 0x7FF, eb = (int)(hiw(bb) >> 20) & 0x7FF, eq = (int)(hiw(bq) >> 20) & 0x7FF;
-  if ((unsigned)(ea - 1) >= 2046u || (unsigned)(eb - 1) >= 2046u || (unsigned)(eq - 3) >= 2040u) return q;
-  const u64 frac = (1ull << 52) - 1, one = 1ull << 52;
-  const u64 ma = ((u64)ba & frac) | one, mb = ((u64)bb & frac) | one, mq = ((u64)bq & frac) | one;
-  // q = mq 2^(eq - 1075): a 2^k = q b + rem with k = 52 or 53 bits between ma and mq mb
-  const int k = ea - eb - eq + 1075;                 // ma 2^k and mq mb on one grid
-  const i64 rem = (i64)((ma << k) - mq * mb);        // |rem| < mb
-  if (2 * rem > (i64)mb) return of_bits(bq + 1);
-  if (-2 * rem > (i64)mb) return of_bits(bq - 1);
-  return q;
+  const u64 mb = ((u64)bb & ((1ull << 52) - 1)) | (1ull << 52);
+  const i64 r = rcp62((unsigned)(mb >> 32), low(bb));
+  const double q = pack61((u64)(r >> 1), 2046 - eb, hiw(bb) & 0x80000000u);
+  const int eq = (int)(hiw(bits(q)) >> 20) & 0x7FF;
+  return round_quotient(q, 1ull << 52, mb, 2046 - eb - eq + 52);
 }
 
 // the pieces of a positive normal a = m 4^k: M = m 2^52 (m in [1, 4)), m in FP32, k
@@ -217,7 +222,12 @@ SF_HD double ssqrt(double a) {
   const i64 y = rsqrt62(M, f);                             // (2^61, 2^62]
   // m y in [1, 2): (M 2^8) y 2^-62 = sqrt(m) 2^60
   const i64 Q = mulhi62(M << 8, y - (y >> 62));
-  return pack61((u64)(Q << 1), 1023 + k, 0u);
+  const i64 bq = bits(pack61((u64)(Q << 1), 1023 + k, 0u));
+  // q on the grid of [1, 2) (2 itself may come out of the rounding), off by less than one
+  // unit: corrected by the remainder M 2^52 - q^2, which the low 64 bits hold
+  const i64 q = (i64)((((u64)bq & ((1ull << 52) - 1)) | (1ull << 52)) << ((int)(hiw(bq) >> 20) - 1023 - k));
+  const i64 rem = (i64)(((u64)M << 52) - (u64)q * (u64)q);
+  return of_bits(bq + (rem > q) - (rem <= -q));
 }
 
 // 1 / sqrt(a)
