@@ -501,8 +501,9 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
     gi_scale = 1.0;
   }
   // S_i = 0 (matter at rest): r = 0 without the contraction
+  const bool rest = is_zero(S[0]) && is_zero(S[1]) && is_zero(S[2]);
   double r = 0.0;
-  if (!is_zero(S[0]) || !is_zero(S[1]) || !is_zero(S[2])) r = t_div(t_sqrt(W * W * gi_scale * s3quad(gi, S, S)), D);
+  if (!rest) r = t_div(t_sqrt(W * W * gi_scale * s3quad(gi, S, S)), D);
   if (p.adiabatic) {
     // "adiabatic" EOS (Sec. III): zero temperature, the energy equation is
     // discarded: the cold recovery from D and S_i alone, the Lorentz factor
@@ -533,8 +534,9 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
     prim_to_cons(p, pr, W, gt, x, q);
     return st;
   }
-  if (is_zero(r) && !p.mlp) {
-    // matter at rest: the bracket is z = 0, its master function vanishes there, w = 1
+  if (rest && !p.mlp) {
+    // matter at rest: the bracket is z = 0, its master function vanishes there, w = 1.  (Momenta so
+    // small that r underflows to zero are not at rest: u_i = S_i / (D h) below.)
     if (p.c2p_stats) {
       atomicAdd(p.c2p_stats + 0, 2ull);
       atomicAdd(p.c2p_stats + 3, 1ull);
