@@ -500,8 +500,9 @@ __device__ inline int cons_to_prim(const DevParams &p, double q[NCONS], double W
     gi.yy *= gi_scale; gi.yz *= gi_scale; gi.zz *= gi_scale;
     gi_scale = 1.0;
   }
-  // S_i = 0 (matter at rest): r = 0 without the contraction
-  const bool rest = is_zero(S[0]) && is_zero(S[1]) && is_zero(S[2]);
+  // S_i = 0 (matter at rest): r = 0 without the contraction; a metric that is not finite makes r NaN
+  const bool rest = is_zero(S[0]) && is_zero(S[1]) && is_zero(S[2]) && is_finite(gi.xx) && is_finite(gi.xy) &&
+                    is_finite(gi.xz) && is_finite(gi.yy) && is_finite(gi.yz) && is_finite(gi.zz);
   double r = 0.0;
   if (!rest) r = t_div(t_sqrt(W * W * gi_scale * s3quad(gi, S, S)), D);
   if (p.adiabatic) {

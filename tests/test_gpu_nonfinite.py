@@ -47,3 +47,16 @@ def test_tiny_momenta_are_not_rest(adiabatic):
     for f in (1, 3):
         assert np.all(np.abs(a[f] - b[f]) <= 1e-14 * np.abs(b[f])) and np.all(b[f] != 0.0)
 
+
+@pytest.mark.parametrize("value", [np.nan])
+@pytest.mark.parametrize("field", [1, 2, 5, 6])
+@pytest.mark.parametrize("adiabatic", [0, 1])
+def test_recovery_in_a_broken_metric(adiabatic, field, value):
+    """Matter at rest in a cell whose h_ij is not finite: the same cells, and only those, lose their
+    primitives and say so in their status."""
+    def change(raw):
+        raw[field, G + 3:G + 5, G + 10:G + 20] = value
+    a, b, sa, sb = _recover(adiabatic, change)
+    assert np.array_equal(sa, sb)
+    for f in range(6):
+        assert np.array_equal(np.isfinite(a[f]), np.isfinite(b[f])), f
