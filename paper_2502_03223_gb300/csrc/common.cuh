@@ -444,7 +444,8 @@ __device__ double illinois_from(const DevParams &p, double a, double fa, double 
       if (last == +1) fb *= 0.5;
       last = +1;
     }
-    if (!less_any(p.c2p_tol * fmax(fabs(c), 1e-30), fabs(b - a))) return c;
+    const double width = fabs(b - a);
+    if (!is_nan(width) && !less_any(p.c2p_tol * fmax(fabs(c), 1e-30), width)) return c;
   }
   *ok = 0;
   return c;

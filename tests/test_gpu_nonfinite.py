@@ -48,7 +48,7 @@ def test_tiny_momenta_are_not_rest(adiabatic):
         assert np.all(np.abs(a[f] - b[f]) <= 1e-14 * np.abs(b[f])) and np.all(b[f] != 0.0)
 
 
-@pytest.mark.parametrize("value", [np.nan])
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
 @pytest.mark.parametrize("field", [1, 2, 5, 6])
 @pytest.mark.parametrize("adiabatic", [0, 1])
 def test_recovery_in_a_broken_metric(adiabatic, field, value):
