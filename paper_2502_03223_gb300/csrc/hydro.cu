@@ -44,6 +44,20 @@ __device__ __forceinline__ double face6(const double *u, int s) {
   return __longlong_as_double(sb + ((long long)(E - fx::kGrid - 8) << 52));
 }
 
+// The largest exponent of values, as the top half of their patterns shifted by
+// the sign: kTopInf and above is an infinity or NaN.
+constexpr unsigned kTopInf = 0xFFE00000u;
+__device__ __forceinline__ unsigned top_of(const double *u) {
+  return (unsigned)__double2hiint(*u) << 1;
+}
+__device__ __forceinline__ unsigned stencil_top(const double *u, int s) {      // of the six values of face6
+  unsigned t = top_of(u);
+#pragma unroll
+  for (int n = -2; n <= 3; ++n)
+    if (n != 0) t = max(t, top_of(u + n * s));
+  return t;
+}
+
 // Face j+1/2 (dir 0, stride 1) or k+1/2 (dir 1, stride px) of cell (j, k):
 // reconstruction, metric at the face and the flux, FP64.
 // The flux of the face from its reconstructed states pl (cell side), pr
@@ -67,24 +81,33 @@ __device__ inline void flux_states_f64(const Lev &L, const DevParams &p, const d
   // Equal states at rest (the atmosphere, most faces of a star's grid): the
   // flux of that state, f - v_int q, in closed form.  With u_i = 0 only the
   // pressure and the shift are left, and the tetrad's factors cancel:
-  // (D, E) -beta^n / W^3, normal momentum alpha P / W^3.  3.65 -> 3.20 ms per
-  // direction and step of the migration star 5 x 512^2.
+  // (D, E) -beta^n / W^3, normal momentum alpha P / W^3.  A value that is not
+  // finite in what drops out (h_ij, the transverse shift) leaves the general
+  // form, whose result it makes NaN.
   long long diff = 0;
 #pragma unroll
   for (int v = 0; v < 5; ++v) diff |= fx::bits(pl[v]) ^ fx::bits(pr[v]);
 #pragma unroll
   for (int v = 1; v < 4; ++v) diff |= fx::bits(pl[v]) << 1;
   if (diff == 0) {
+    unsigned top = 0;
+#pragma unroll
+    for (int f = 0; f < 6; ++f) top = max(top, stencil_top(U + (size_t)(fHXX + f) * P + id, s));
+    top = max(top, stencil_top(U + (size_t)fBY * P + id, s));
+    top = max(top, stencil_top(U + (size_t)(DIR == 0 ? fBZ : fBX) * P + id, s));
     const double bn = face6(U + (size_t)(DIR == 0 ? fBX : fBZ) * P + id, s);
-    const double iW = t_rcp(W), iW3 = iW * iW * iW;
     const double rho = pl[0], pc = eos_pc(p, rho), Pp = p.adiabatic ? pc : pl[4];
-    const double a = -bn * iW3;
-    out[0] = a * rho;
-    out[4] = a * (rho * (1.0 + eos_ec(p, rho)) + (Pp - pc) * p.ith1);
-    out[1] = out[2] = out[3] = 0.0;
-    out[DIR == 0 ? 1 : 3] = alpha * iW3 * Pp;
-    *fb = 0;
-    return;
+    if (top < kTopInf && is_finite(alpha) && !is_zero(alpha) && is_finite(W) && is_finite(bn) &&
+        (unsigned)__double2hiint(rho) - 0x00100000u < 0x7FE00000u && is_finite(Pp)) {
+      const double iW = t_rcp(W), iW3 = iW * iW * iW;
+      const double a = -bn * iW3;
+      out[0] = a * rho;
+      out[4] = a * (rho * (1.0 + eos_ec(p, rho)) + (Pp - pc) * p.ith1);
+      out[1] = out[2] = out[3] = 0.0;
+      out[DIR == 0 ? 1 : 3] = alpha * iW3 * Pp;
+      *fb = 0;
+      return;
+    }
   }
   double beta[3];
 #pragma unroll
@@ -564,8 +587,24 @@ __device__ __forceinline__ void hydro_rhs_cell(const Lev &L, const DevParams &p,
   if constexpr (sizeof(T) == 8) {
     if (u[0] == 0.0 && u[1] == 0.0 && u[2] == 0.0) {
       // matter at rest (the atmosphere): only the pressure, its trace with
-      // K_ij = (At_ij + gt_ij K / 3) / W^2 and the gradients of alpha and W are left:
-      // 2.44 -> 1.90 ms per step of the migration star 5 x 512^2
+      // K_ij = (At_ij + gt_ij K / 3) / W^2 and the gradients of alpha and W are left.
+      // A value that is not finite in what drops out (beta^i, the differences of
+      // beta^i and h_ij) leaves the general form, whose result it makes NaN.
+      unsigned top = top_of(U + (size_t)fBY * P + id);
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        const int f = q < 6 ? fHXX + q : fBX + q - 6;
+        if (use_ds) {
+          // the dissipation of the field, which takes every value its differences take
+          top = max(top, top_of(reinterpret_cast<const double *>(DS) + (size_t)(DS_AK + f) * P + id));
+        } else {
+#pragma unroll
+          for (int n = 1; n <= 3; ++n)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+              top = max(top, max(top_of(U + (size_t)f * P + id + n * st[e]), top_of(U + (size_t)f * P + id - n * st[e])));
+        }
+      }
       const double iW = t_rcp(W), iW3 = iW * iW * iW;
       const double rh = rho * (1.0 + pr[pEPS]) + Pp;
       const double trA = gi.xx * ld(fAXX) + gi.yy * ld(fAYY) + gi.zz * ld(fAZZ)
@@ -574,16 +613,17 @@ __device__ __forceinline__ void hydro_rhs_cell(const Lev &L, const DevParams &p,
       const double aP = al * Pp, c3 = -3.0 * aP * iW;
       double s[2];
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        s[e] = iW3 * ((Pp - rh) * d1(fAL, e) + c3 * d1(fW, e));
+      for (int e = 0; e < 2; ++e) s[e] = iW3 * ((Pp - rh) * d1(fAL, e) + c3 * d1(fW, e));
+      const double sE = iW3 * aP * (trA + K);
+      if (top < kTopInf && is_finite(s[0]) && is_finite(s[1]) && is_finite(sE) && !is_zero(al)) {
+        double *rq = L.rhsq + id;
+        rq[0] = -div[0];
+        rq[P] = s[0] + (cyl ? t_div(aP * iW3, xd) : 0.0) - div[1];
+        rq[2 * P] = -div[2];
+        rq[3 * P] = s[1] - div[3];
+        rq[4 * P] = sE - div[4];
+        return;
       }
-      double *rq = L.rhsq + id;
-      rq[0] = -div[0];
-      rq[P] = s[0] + (cyl ? t_div(aP * iW3, xd) : 0.0) - div[1];
-      rq[2 * P] = -div[2];
-      rq[3 * P] = s[1] - div[3];
-      rq[4 * P] = iW3 * aP * (trA + K) - div[4];
-      return;
     }
   }
   const T w = t_sqrt(T(1) + W * W * s3quad(gi, u, u));

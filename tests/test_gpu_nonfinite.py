@@ -60,3 +60,56 @@ def test_recovery_in_a_broken_metric(adiabatic, field, value):
     assert np.array_equal(sa, sb)
     for f in range(6):
         assert np.array_equal(np.isfinite(a[f]), np.isfinite(b[f])), f
+
+
+def _at_rest(evolve):
+    """A star at rest with a mildly varying metric and shift (16 x 12 cells), and its PRIM_METRIC planes."""
+    cfg, tov = W.tov_config("rest", rho_c=1.28e-3, n_levels=1, N=16, dx_fine=0.9, rk=0)
+    cfg = dataclasses.replace(cfg, nz=12, evolve_spacetime=evolve)
+    d = W.tov_level_data(cfg, tov, 0)
+    d[:25] += W.random_metric_perturbation(cfg, 0, np.random.default_rng(8), amp=1e-2)
+    return cfg, d
+
+
+def _rates(field, value):
+    """Rates of the conserved variables, GPU and oracle, with one primitive set to `value`."""
+    cfg, d = _at_rest(0)
+    d[25 + field, G + 6, G + 7] = value
+    g, o = S.Sacra(cfg), O.Oracle(cfg)
+    g.set_initial_data(0, S.PRIM_METRIC, d)
+    g.fill(0, cfg.dt)
+    g.rk_stage(0, cfg.dt)
+    o.set_level(0, 0, d)
+    o.fill(0, cfg.dt)
+    o.stage(0, cfg.dt)
+    return (np.stack([g.read(0, S.RHS, f, padded=False) for f in range(25, 30)]),
+            np.stack([o.read(0, 3, f)[G:G + cfg.nz, G:G + cfg.nx] for f in range(25, 30)]))
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("evolve,field", [(e, f) for e in (0, 1) for f in (0, 1, 3, 5, 9, 13, 18, 19, 20, 21)
+                                          if (e, f) != (0, 20)])
+def test_hydro_rates_in_a_broken_metric(evolve, field, value):
+    """Matter at rest around one metric value that is not finite: the rates of the conserved variables
+    are lost in the cells whose faces and sources read it, and in no other."""
+    cfg, d = _at_rest(evolve)
+    d[field, G + 6, G + 7] = value
+    g, o = S.Sacra(cfg), O.Oracle(cfg)
+    g.set_initial_data(0, S.PRIM_METRIC, d)
+    g.fill(0, cfg.dt)
+    g.rk_stage(0, cfg.dt)
+    o.set_level(0, 0, d)
+    o.fill(0, cfg.dt)
+    o.stage(0, cfg.dt)
+    for f in range(25, 30):
+        a = np.isfinite(g.read(0, S.RHS, f, padded=False))
+        b = np.isfinite(o.read(0, 3, f)[G:G + cfg.nz, G:G + cfg.nx])
+        assert np.array_equal(a, b), (f, np.argwhere(a != b)[:8])
+
+
+@pytest.mark.parametrize("field,value", [(0, np.nan), (0, np.inf), (4, np.nan), (4, np.inf)])
+def test_hydro_rates_around_broken_matter(field, value):
+    """A density or pressure that is not finite in matter at rest: the same rates are lost."""
+    a, b = _rates(field, value)
+    assert np.array_equal(np.isfinite(a), np.isfinite(b))
+
