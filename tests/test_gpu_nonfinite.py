@@ -113,3 +113,12 @@ def test_hydro_rates_around_broken_matter(field, value):
     a, b = _rates(field, value)
     assert np.array_equal(np.isfinite(a), np.isfinite(b))
 
+
+@pytest.mark.parametrize("field,value", [(1, np.nan), (2, np.nan), (3, np.nan), (1, np.inf), (3, -np.inf)])
+def test_broken_velocities_reach_their_neighbours(field, value):
+    """A velocity that is not finite in matter at rest: every rate of the cell and of the four next to it
+    is lost (both states of a face between them are made with it), beyond them at most what the oracle loses."""
+    a, b = _rates(field, value)
+    for k, j in ((6, 7), (5, 7), (7, 7), (6, 6), (6, 8)):
+        assert not np.isfinite(a[:, k, j]).any(), (k, j)
+    assert not (~np.isfinite(a) & np.isfinite(b)).any()
