@@ -261,11 +261,14 @@ SF_HD void z4c_pass_b(const Z4cPar<T> &p, FU U, F1 D1, F2 D2, FA AK, FP PR, FS s
 
   // ---- matter
   const T PI = T(3.14159265358979323846L);
-  T E, SE, Si[3] = {T(0), T(0), T(0)};              // E, tr S + E, S_i
+  T E, SE, Si[3];                                   // E, tr S + E, S_i
   {
     const T P = PR(pP);
     const T ud[3] = {PR(pUX), PR(pUY), PR(pUZ)};
     const T rh = PR(pRHO) * (T(1) + PR(pEPS)) + P;
+    const T none = T(0) * rh;                       // NaN where rho, eps or P is not finite
+    Si[0] = Si[1] = Si[2] = none;
+    trX += none;
     E = rh - P;
     SE = rh + T(2) * P;
     if (ud[0] != T(0) || ud[1] != T(0) || ud[2] != T(0)) {

@@ -122,3 +122,23 @@ def test_broken_velocities_reach_their_neighbours(field, value):
     for k, j in ((6, 7), (5, 7), (7, 7), (6, 6), (6, 8)):
         assert not np.isfinite(a[:, k, j]).any(), (k, j)
     assert not (~np.isfinite(a) & np.isfinite(b)).any()
+
+
+@pytest.mark.parametrize("field,value", [(25, np.nan), (25, np.inf), (29, np.nan), (29, np.inf), (26, np.nan), (2, np.inf),
+                                         (8, np.nan), (13, np.inf), (15, np.nan), (17, np.inf), (23, np.inf)])
+def test_metric_rates_around_a_broken_value(field, value):
+    """One metric value or primitive that is not finite: the rates of the metric are lost in the cells
+    where the oracle loses them."""
+    cfg, d = _at_rest(1)
+    d[field, G + 6, G + 7] = value
+    g, o = S.Sacra(cfg), O.Oracle(cfg)
+    g.set_initial_data(0, S.PRIM_METRIC, d)
+    g.fill(0, cfg.dt)
+    g.rk_stage(0, cfg.dt)
+    o.set_level(0, 0, d)
+    o.fill(0, cfg.dt)
+    o.stage(0, cfg.dt)
+    for f in range(25):
+        a = np.isfinite(g.read(0, S.RHS, f, padded=False))
+        b = np.isfinite(o.read(0, 3, f)[G:G + cfg.nz, G:G + cfg.nx])
+        assert np.array_equal(a, b), (f, np.argwhere(a != b)[:8])
