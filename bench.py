@@ -58,10 +58,11 @@ UNIT = "cell-updates/s"
 # star's second step: they include what the data decide (faces between equal
 # states take the state's own flux, matter at rest skips its Lorentz factor,
 # the recovery's iteration counts), counted on the formulation that ran all of it
-# in FP64.  The kernels now run most of this work on the integer units (sums in
-# block fixed point, quotients and roots) or in closed form (matter at rest, slow
-# flow), so these are FP64-equivalent operations and a fraction of the FP64 peak
-# may pass 1.  Units: a cell of the update region; a face
+# in FP64.  The kernels run a part of this work on the integer units (stencil and
+# face sums, quotients and roots), leave a part out by identities (pointwise Z4c)
+# or closed forms (matter at rest, slow flow), so these are FP64-equivalent
+# operations of the method: a rate of work done, not a bound, and the fraction of
+# the FP64 peak may pass 1.  Units: a cell of the update region; a face
 # for the flux kernels; a cell of the plane patch for the cartoon kernel.
 METHOD_FLOPS = {
     "k_z4c_derivs": 2139.0, "k_cartoon": 591.0, "k_z4c_point": 2001.0, "k_flux_x": 508.0,
@@ -686,8 +687,8 @@ def run_native(args, dist, rank, ws, local):
                 "peak_source": "FP64 FMA probe measured in this run (nominal %.2f TFLOP/s); of measured"
                                % NOMINAL_FP64_TFLOPS,
                 "method_flops_per_unit": METHOD_FLOPS[dom],
-                "work": "FP64-equivalent operations of the method; most of them run on the integer units, "
-                        "so a fraction of the FP64 peak may pass 1", "avg_launch_ms": avg_s * 1e3,
+                "work": "FP64-equivalent operations of the method, a part of which runs on the integer units or is left "
+                        "out by identities: frac is a rate of work, not a distance to a limit, and may pass 1", "avg_launch_ms": avg_s * 1e3,
                 "units_per_launch": units_per_launch,
                 "kernel_share": {k: round(v[0] / sum(x[0] for x in kern.values()), 4) for k, v in
                                  sorted(kern.items(), key=lambda kv: -kv[1][0])[:10]},

@@ -301,17 +301,16 @@ __device__ __forceinline__ void enforce_algebraic(double &W, double h[6], double
 // and primitive recovery.  Ust = stage state read (Un at stage 0, Us after);
 // the result is written to Us.
 //
-// The update is bound by the latency of its ~100 loads per cell (30 fields of
-// three registers) and by the FP64 pipe, not by its bytes.  The fields go
+// The update is bound by the FP64 pipe and by the latency of its ~100 loads
+// per cell (30 fields of three registers), not by its bytes.  The fields go
 // through in groups whose loads are all in flight together and whose indices
-// are compile-time constants, so that no field waits in local memory: the
-// eleven fields that are only combined, then those of the algebraic
-// constraints, then the conserved ones.  Five blocks per SM (four and six are
-// within 2 %).  With one field's loads at a time and three blocks per SM it
-// took 5.3 ms per step of the migration star (5 x 512^2), 4.1 with groups of
-// five fields through local memory, 2.9 now (with the recovery's closed forms
-// for matter at rest and slow flow, common.cuh); 42 -> 26 ms per coarse step
-// of 7 x 1024^2.
+// are compile-time constants: the eleven fields that are only combined, then
+// those of the algebraic constraints, then the conserved ones.  Five blocks per
+// SM, which cost 400 bytes of spills per thread (four and six blocks are within
+// 2 %).  3.0 ms per step of the migration star 5 x 512^2; with one field's loads
+// at a time and three blocks per SM 5.3, with groups of five fields through a
+// local array 4.1, before the recovery's closed forms for matter at rest and
+// slow flow (common.cuh).  26 ms per coarse step of 7 x 1024^2 (42 before them).
 constexpr int kRkBlocks = 5;
 struct RkTerm {
   double un, kk, aux;
