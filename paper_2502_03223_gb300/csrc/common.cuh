@@ -223,14 +223,17 @@ __device__ __forceinline__ float t_rcp(float a) { return 1.0f / a; }
 __device__ __forceinline__ float t_sqrt(float a) { return sqrtf(a); }
 __device__ __forceinline__ float t_rsqrt(float a) { return rsqrtf(a); }
 
-// d^(-1/3) by one third-order (Householder) step from an FP32 seed:
+// d^(-1/3) by one third-order (Householder) step from an FP32 seed y0:
 // e = 1 - d y0^3, y0 (1 + e/3 + 2/9 e^2); the next term is 14/81 e^3 < 2^-60.
-// Six FP64 operations (rcbrt takes the time of sixteen).
+// y0^2 is exact and e is formed from d y0^2 in two parts, so that no rounding
+// but the last one counts (0.501 ulp).  Nine FP64 operations (rcbrt takes the
+// time of sixteen).
 __device__ __forceinline__ double t_rcbrt(double d) {
   const int hi = __double2hiint(d);
   if (hi < 0x3E000000 || hi >= 0x42000000) return rcbrt(d);   // a determinant far from 1, or not a positive number
   const double y0 = f64_of(exp2f(log2f(f32_of(d)) * (-1.0f / 3.0f)));
-  const double e = fma(-d, y0 * y0 * y0, 1.0);
+  const double p = y0 * y0, t = __dmul_rn(d, p);
+  const double e = fma(-fma(d, p, -t), y0, fma(-t, y0, 1.0));
   return fma(y0 * e, fma(e, 2.0 / 9.0, 1.0 / 3.0), y0);
 }
 
